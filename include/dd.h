@@ -154,7 +154,14 @@ dd_status dd_autotune(dd_plan_t plan, const void *in, dd_dtype dtype, int64_t in
  * and a count of tile rounds says it finishes earlier, the DMs of that tile
  * run as a second launch on a library-owned stream: it waits for an event
  * recorded on `stream` before the call's work, and `stream` waits for its
- * completion, so every later operation on `stream` sees the whole plane. */
+ * completion, so every later operation on `stream` sees the whole plane.
+ * uint8 beams of the preferred tile shape (4 DMs x 8 words per thread, 12 DM
+ * warps, 8-channel stages) whose neighbouring channels' shifts differ little
+ * run in a kernel of its own tiles (64 DMs x 1024 samples) that sums groups of
+ * channels once per shift pattern, where a count of tile rounds says it
+ * finishes earlier; the sums are the same.  Its table (2.5 KB per 64 DMs and 8
+ * channels) is built on the first such call, outside `stream`, and held with
+ * the plan; without memory for it the direct kernel runs. */
 dd_status dd_execute(dd_plan_t plan, const void *in, dd_dtype dtype, int64_t in_pitch,
                      int64_t nsamp_in, float *out, int64_t out_pitch, int64_t nsamp_out,
                      void *stream);
@@ -377,7 +384,9 @@ typedef struct dd_batch_s *dd_batch_t;
  * an atomic counter.  The launch (and the reset of the counter before it) is
  * captured once into a CUDA graph and replayed by later
  * dd_batch_execute calls (re-captured after dd_batch_set_io or a tile change).
- * All beams share one tile shape (dd_batch_set_tiles / dd_batch_autotune).
+ * All beams share one tile shape (dd_batch_set_tiles / dd_batch_autotune);
+ * with the preferred uint8 shape, beams that gain by channel groups (see
+ * dd_execute) run in a second launch beside it.
  * plans[i] must outlive the batch; the batch owns its device descriptors and
  * counters. */
 dd_status dd_batch_create(const dd_plan_t *plans, int nbeams, dd_dtype dtype,

@@ -8,6 +8,10 @@
 // cost (channel count) first -- and the kernel's producer warps claim global
 // tile numbers from an atomic counter, so big beams start first and small
 // tiles fill the tail.
+//
+// Beams that gain by channel groups (dd_group.h) go to a second launch that
+// runs beside the persistent one, on a forked stream: its tiles take the SMs
+// that the persistent CTAs leave.
 #include <cuda_runtime_api.h>
 
 #include <algorithm>
@@ -16,6 +20,7 @@
 #include <string>
 #include <vector>
 
+#include "dd_group.h"
 #include "dd_internal.h"
 #include "dd_kargs.h"
 
@@ -45,7 +50,12 @@ struct dd_batch_s {
     dd::BeamArgs *d_beams = nullptr;
     int *d_counter = nullptr;
     int *d_status = nullptr;
-    dd::KArgs args{};
+    dd::KArgs args{};        // direct launch (args.nbeams == 0: none)
+    dd::GroupBeam *d_gbeams = nullptr;
+    dd::GroupArgs gargs{};   // grouped launch (gargs.nbeams == 0: none)
+    unsigned ggrid = 0;
+    cudaStream_t side = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
     unsigned grid = 0;
     int threads = 0, smem = 0;
     int64_t total_tiles = 0;
@@ -123,15 +133,25 @@ dd_status prepare(dd_batch_s *b) {
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
         return b->beams[x].plan->nchan > b->beams[y].plan->nchan;
     });
-    std::vector<dd::BeamArgs> desc(b->beams.size());
-    int64_t tile0 = 0;
+    std::vector<dd::BeamArgs> desc;
+    std::vector<dd::GroupBeam> gdesc;
+    int64_t tile0 = 0, gtile0 = 0;
     for (size_t k = 0; k < order.size(); ++k) {
         BatchBeam &bb = b->beams[order[k]];
         dd::DevTables *dt = nullptr;
         dd_status st = dd::device_tables(bb.plan, &dt);
         if (st != DD_OK)
             return st;
-        dd::BeamArgs &d = desc[k];
+        dd::GroupShape gs;
+        if (dd::group_shape(bb.plan, b->dtype, bb.g, *dt, bb.nsamp_out, false, &gs)) {
+            gdesc.push_back(dd::group_beam(gs, *dt, bb.in, bb.in_pitch, bb.nsamp_in, bb.out,
+                                           bb.out_pitch, bb.nsamp_out));
+            gdesc.back().tile_begin = gtile0;
+            gtile0 += dd::group_tiles(gs, bb.nsamp_out);
+            continue;
+        }
+        desc.emplace_back();
+        dd::BeamArgs &d = desc.back();
         d.in = static_cast<const uint8_t *>(bb.in);
         d.in_pitch_b = bb.in_pitch * elem;
         d.nsamp_in = bb.nsamp_in;
@@ -150,6 +170,7 @@ dd_status prepare(dd_batch_s *b) {
     }
     if (!b->d_beams) {
         if (cudaMalloc((void **)&b->d_beams, sizeof(dd::BeamArgs) * b->beams.size()) != cudaSuccess ||
+            cudaMalloc((void **)&b->d_gbeams, sizeof(dd::GroupBeam) * b->beams.size()) != cudaSuccess ||
             cudaMalloc((void **)&b->d_counter, sizeof(int)) != cudaSuccess ||
             cudaMalloc((void **)&b->d_status, sizeof(int)) != cudaSuccess) {
             cudaGetLastError();
@@ -158,20 +179,32 @@ dd_status prepare(dd_batch_s *b) {
         cudaMemset(b->d_status, 0, sizeof(int));
     }
     if (cudaMemcpy(b->d_beams, desc.data(), sizeof(dd::BeamArgs) * desc.size(),
+                   cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(b->d_gbeams, gdesc.data(), sizeof(dd::GroupBeam) * gdesc.size(),
                    cudaMemcpyHostToDevice) != cudaSuccess)
         return fail(DD_ERR_CUDA, "batch descriptor upload failed");
-    if (tile0 > 0x7fffffffLL)
+    if (!gdesc.empty() && !desc.empty() && !b->side &&
+        (cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking) != cudaSuccess ||
+         cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess ||
+         cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming) != cudaSuccess))
+        return fail(DD_ERR_CUDA, "batch stream creation failed");
+    if (tile0 > 0x7fffffffLL || gtile0 > 0x7fffffffLL)
         return fail(DD_ERR_INVALID, "too many tiles in one batch");
     int nsm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     b->total_tiles = tile0;
+    b->ggrid = (unsigned)gtile0;
+    b->gargs = dd::GroupArgs{};
+    b->gargs.beams = b->d_gbeams;
+    b->gargs.nbeams = (int)gdesc.size();
+    b->gargs.status = b->d_status;
     b->grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(tile0, nsm > 0 ? nsm : 1));
     b->threads = g0.threads;
     b->smem = (int)smem_for(nst);
     dd::KArgs &a = b->args;
     a = dd::KArgs{};
     a.beams = b->d_beams;
-    a.nbeams = (int)b->beams.size();
+    a.nbeams = (int)desc.size();
     a.total_tiles = tile0;
     a.tile_counter = b->d_counter;
     a.dm_warps = b->tiles.dm_warps;
@@ -187,21 +220,42 @@ dd_status prepare(dd_batch_s *b) {
     return DD_OK;
 }
 
-// The tile counter reset, then the persistent de-dispersion launch.
+// The tile counter reset and the persistent launch of the direct beams; the
+// grouped beams' launch beside it.
 dd_status enqueue(dd_batch_s *b, cudaStream_t s, bool count = true) {
-    cudaError_t e = cudaMemsetAsync(b->d_counter, 0, sizeof(int), s);
-    if (e != cudaSuccess)
-        return fail(DD_ERR_CUDA, std::string("batch counter reset: ") + cudaGetErrorString(e));
-    const int dthr = b->tiles.dm_per_thread, nw = b->tiles.words_per_thread;
-    switch (b->dtype) {
-    case DD_U8: e = dd::launch_kernel_u8(b->args, b->grid, b->threads, b->smem, s, dthr, nw); break;
-    case DD_F16: e = dd::launch_kernel_f16(b->args, b->grid, b->threads, b->smem, s, dthr, nw); break;
-    case DD_F32: e = dd::launch_kernel_f32(b->args, b->grid, b->threads, b->smem, s, dthr, nw); break;
+    const bool direct = b->args.nbeams > 0, grouped = b->gargs.nbeams > 0;
+    const bool both = direct && grouped;
+    cudaError_t e = cudaSuccess;
+    if (both) {
+        e = cudaEventRecord(b->fork, s);
+        if (e == cudaSuccess)
+            e = cudaStreamWaitEvent(b->side, b->fork, 0);
+        if (e != cudaSuccess)
+            return fail(DD_ERR_CUDA, std::string("batch fork: ") + cudaGetErrorString(e));
+    }
+    if (direct) {
+        e = cudaMemsetAsync(b->d_counter, 0, sizeof(int), s);
+        if (e != cudaSuccess)
+            return fail(DD_ERR_CUDA, std::string("batch counter reset: ") + cudaGetErrorString(e));
+        const int dthr = b->tiles.dm_per_thread, nw = b->tiles.words_per_thread;
+        switch (b->dtype) {
+        case DD_U8: e = dd::launch_kernel_u8(b->args, b->grid, b->threads, b->smem, s, dthr, nw); break;
+        case DD_F16: e = dd::launch_kernel_f16(b->args, b->grid, b->threads, b->smem, s, dthr, nw); break;
+        case DD_F32: e = dd::launch_kernel_f32(b->args, b->grid, b->threads, b->smem, s, dthr, nw); break;
+        }
+    }
+    if (grouped && e == cudaSuccess)
+        e = dd::launch_group(b->gargs, b->ggrid, both ? b->side : s);
+    if (both) {
+        if (e == cudaSuccess)
+            e = cudaEventRecord(b->join, b->side);
+        if (e == cudaSuccess)
+            e = cudaStreamWaitEvent(s, b->join, 0);
     }
     if (e != cudaSuccess)
         return fail(DD_ERR_CUDA, std::string("batch kernel launch: ") + cudaGetErrorString(e));
     if (count)
-        dd::count_launch(1);
+        dd::count_launch((direct ? 1 : 0) + (grouped ? 1 : 0));
     return DD_OK;
 }
 
@@ -239,8 +293,15 @@ void dd_batch_destroy(dd_batch_t b) {
     cudaDeviceSynchronize();
     drop_graph(b);
     cudaFree(b->d_beams);
+    cudaFree(b->d_gbeams);
     cudaFree(b->d_counter);
     cudaFree(b->d_status);
+    if (b->fork)
+        cudaEventDestroy(b->fork);
+    if (b->join)
+        cudaEventDestroy(b->join);
+    if (b->side)
+        cudaStreamDestroy(b->side);
     if (b->capture)
         cudaStreamDestroy(b->capture);
     delete b;

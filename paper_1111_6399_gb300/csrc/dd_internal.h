@@ -6,6 +6,7 @@
 
 #include <cstdint>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -99,6 +100,8 @@ struct Geometry {
     int threads = 0;      // consumer warps + one producer warp + builder warps
 };
 
+struct GroupShape;  // dd_group.h
+
 }  // namespace dd
 
 struct dd_plan_s {
@@ -116,6 +119,7 @@ struct dd_plan_s {
     std::map<uint64_t, dd::Geometry> geo;  // per (dtype, tiles) key
     // Remainder-DM launch per (dtype, tiles) key: (found, geometry).
     std::map<uint64_t, std::pair<bool, dd::Geometry>> tail_geo;
+    std::map<int, std::shared_ptr<dd::GroupShape>> group;  // grouped execution, per device
 };
 
 namespace dd {
@@ -167,7 +171,9 @@ dd_status tail_geometry(dd_plan_s *p, dd_dtype t, const Geometry &g, bool *found
 // Device tables for the current device, uploaded on first use.
 dd_status device_tables(dd_plan_s *p, DevTables **out);
 
-// Launch the de-dispersion kernel (dd_kernel_*.cu) for one beam on stream.
+// Launch the de-dispersion of one beam on stream: the grouped kernel
+// (dd_group.cu; unless `grouped` is false) where it is expected to be faster,
+// else the direct kernel (dd_kernel_*.cu).
 // With split_tail, the DMs of a last DM tile that is at most half full run
 // as a second launch with their own tile shape, on a library stream forked
 // from and joined back into `stream`, so its CTAs fill the SMs the first
@@ -176,9 +182,12 @@ dd_status device_tables(dd_plan_s *p, DevTables **out);
 dd_status launch_dedisperse(dd_plan_s *p, const Geometry &g, const DevTables &dt,
                             const void *in, dd_dtype dtype, int64_t in_pitch, int64_t nsamp_in,
                             float *out, int64_t out_pitch, int64_t nsamp_out, void *stream,
-                            bool split_tail = true);
+                            bool split_tail = true, bool grouped = true);
 
 void count_launch(int n = 1);
+
+// SMs of a device (0 if unknown).
+int sm_count(int dev);
 
 // Boxcar search accumulators: clear them (dd_detect.cu), and turn them into
 // mean, std, S/N and peak t for an integer-valued plane.

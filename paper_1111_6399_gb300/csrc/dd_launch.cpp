@@ -9,6 +9,7 @@
 #include <string>
 #include <vector>
 
+#include "dd_group.h"
 #include "dd_internal.h"
 #include "dd_kargs.h"
 
@@ -36,19 +37,6 @@ constexpr double kTailCost = 1.4;
 // Shared memory of an SM available to resident CTAs (228 KB less 1 KB per
 // CTA the system reserves).
 constexpr int kSmemPerSm = 233472;
-
-int sm_count(int dev) {
-    static int cached[64] = {0};
-    if (dev < 0 || dev >= 64)
-        return 0;
-    if (cached[dev] == 0) {
-        int n = 0;
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-            return 0;
-        cached[dev] = n;
-    }
-    return cached[dev];
-}
 
 int resident(const Geometry &g) { return std::max(1, kSmemPerSm / (g.smem + 1024)); }
 
@@ -142,6 +130,19 @@ cudaError_t enqueue(dd_plan_s *p, const Geometry &g, const DevTables &dt, int d0
 
 }  // namespace
 
+int sm_count(int dev) {
+    static int cached[64] = {0};
+    if (dev < 0 || dev >= 64)
+        return 0;
+    if (cached[dev] == 0) {
+        int n = 0;
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return 0;
+        cached[dev] = n;
+    }
+    return cached[dev];
+}
+
 dd_status launch_dedisperse_detect(dd_plan_s *p, const Geometry &g, const DevTables &dt,
                                    const void *in, int64_t in_pitch, int64_t nsamp_in,
                                    float *out, int64_t out_pitch, int64_t nsamp_out,
@@ -166,9 +167,29 @@ dd_status launch_dedisperse_detect(dd_plan_s *p, const Geometry &g, const DevTab
 dd_status launch_dedisperse(dd_plan_s *p, const Geometry &g, const DevTables &dt, const void *in,
                             dd_dtype dtype, int64_t in_pitch, int64_t nsamp_in, float *out,
                             int64_t out_pitch, int64_t nsamp_out, void *stream,
-                            bool split_tail) {
+                            bool split_tail, bool grouped) {
     if (nsamp_out == 0)
         return DD_OK;
+    GroupShape gs;
+    if (grouped && group_shape(p, dtype, g, dt, nsamp_out, true, &gs)) {
+        cudaStream_t s = static_cast<cudaStream_t>(stream);
+        const int64_t tiles = group_tiles(gs, nsamp_out);
+        if (tiles > 0x7fffffffLL)
+            return fail(DD_ERR_INVALID, "too many tiles for one launch");
+        GroupArgs a{};
+        a.beam0 = group_beam(gs, dt, in, in_pitch, nsamp_in, out, out_pitch, nsamp_out);
+        a.nbeams = 1;
+        a.status = dt.status;
+        if (g_prof_start)
+            cudaEventRecord(g_prof_start, s);
+        const cudaError_t e = launch_group(a, (unsigned)tiles, s);
+        if (e != cudaSuccess)
+            return fail(DD_ERR_CUDA, std::string("kernel launch failed: ") + cudaGetErrorString(e));
+        if (g_prof_stop)
+            cudaEventRecord(g_prof_stop, s);
+        count_launch(1);
+        return DD_OK;
+    }
     const int64_t ntile_t = (nsamp_out + g.t_cta - 1) / g.t_cta;
     if (ntile_t * g.ntile_d > 0x7fffffffLL)
         return fail(DD_ERR_INVALID, "too many tiles for one launch");

@@ -17,6 +17,7 @@
 #include <numeric>
 #include <new>
 
+#include "dd_group.h"
 #include "dd_internal.h"
 
 namespace {
@@ -372,6 +373,7 @@ void dd_plan_destroy(dd_plan_t p) {
         cudaFree(kv.second.status);
         cudaFree(kv.second.det_cnt);
     }
+    dd::group_free(p);
     if (cur >= 0 && !p->dev.empty())
         cudaSetDevice(cur);
     delete p;
