@@ -68,7 +68,7 @@ extern "C" dd_status dd_execute(dd_plan_t p, const void *in, dd_dtype dtype, int
     if (!in || !out || !aligned16(in) || !aligned16(out))
         return fail(DD_ERR_INVALID, "in and out must be non-NULL and 16-byte aligned");
     dd::Geometry g;
-    if ((st = dd::plan_geometry(p, dtype, &g)) != DD_OK)
+    if ((st = dd::execution_geometry(p, dtype, nsamp_out, &g)) != DD_OK)
         return st;
     dd::DevTables *dt = nullptr;
     if ((st = dd::device_tables(p, &dt)) != DD_OK)
@@ -120,9 +120,6 @@ extern "C" dd_status dd_execute_host(dd_plan_t p, const void *in_host, dd_dtype 
         return DD_OK;
     if (!in_host || !out_host)
         return fail(DD_ERR_INVALID, "NULL host buffer");
-    dd::Geometry g;
-    if ((st = dd::plan_geometry(p, dtype, &g)) != DD_OK)
-        return st;
     dd::DevTables *dt = nullptr;
     if ((st = dd::device_tables(p, &dt)) != DD_OK)
         return st;
@@ -217,6 +214,9 @@ extern "C" dd_status dd_execute_host(dd_plan_t p, const void *in_host, dd_dtype 
             e = cudaEventRecord(ws.landed[i], s);
         if (e != cudaSuccess)
             return fail(DD_ERR_CUDA, std::string("input copy: ") + cudaGetErrorString(e));
+        dd::Geometry g;
+        if ((st = dd::execution_geometry(p, dtype, nb, &g)) != DD_OK)
+            return st;
         st = dd::launch_dedisperse(p, g, *dt, din, dtype, dpitch_in / elem, nb + S,
                                        ws.out[i], dpitch_out, nb, s);
         if (st != DD_OK)

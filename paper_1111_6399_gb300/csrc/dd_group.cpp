@@ -86,12 +86,13 @@ double group_clocks(const Sample &s, int G) {
     return users + 3.9 * (3 * units + 4.5 * arrays / G + units);
 }
 
-// The direct kernel's clocks per channel and tile of its default shape (48 DMs
-// x 1024 samples): 560 .. 600 measured on the same beams where a 64-DM tile
-// spans up to 430 samples, 729 at 860.
-double direct_clocks(double spread) { return 590.0 + 0.32 * std::max(0.0, spread - 430.0); }
-// Prologue and epilogue of a tile.
+// The direct kernel's times are measured where a 64-DM tile spans up to 430
+// samples (590 clocks per channel and tile of its preferred shape); wider
+// windows cost it more (729 clocks at 860 samples).
+double spread_factor(double spread) { return 1.0 + 0.32 / 590 * std::max(0.0, spread - 430.0); }
+// Prologue and epilogue of a tile, clocks.
 constexpr double kTileClocks = 10000;
+constexpr double kClocksPerUs = 2070;
 // Grouped execution is taken when it is expected to gain this much: the model
 // is good to about 5 %.
 constexpr double kGain = 0.95;
@@ -101,16 +102,23 @@ constexpr double kGain = 0.95;
 bool group_shape(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &dt,
                  int64_t nsamp_out, bool alone, GroupShape *out) {
     // The preferred tile shape stands for the library's choice; another shape
-    // set by the caller, or narrower ones for very wide DM tiles, run as such.
+    // set by the caller runs as such.
     const dd_tiles pref = default_tiles(DD_U8);
     int dev = 0;
-    if (t != DD_U8 || std::memcmp(&pref, &g.tiles, sizeof(pref)) != 0 ||
+    if (t != DD_U8 || (std::memcmp(&pref, &g.tiles, sizeof(pref)) != 0 && !tiles_open(p, t)) ||
         cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
         return false;
     const int sms = sm_count(dev);
     const int64_t tiles = (nsamp_out + g.t_cta - 1) / g.t_cta * g.ntile_d;
     if (sms <= 0 || (alone && tiles <= sms))
-        return false;  // one round of the smaller direct tiles
+        return false;  // one round of the direct kernel's tiles
+    // Time of the direct kernel: in rounds of tiles over the SMs, or, as one of
+    // many beams, its share of them.
+    double direct = direct_time_us(t, g.tiles, p->nchan, p->ndm, nsamp_out, sms);
+    if (direct < 0)
+        return false;
+    if (!alone)
+        direct *= (double)tiles / sms / (double)((tiles + sms - 1) / sms);
     std::lock_guard<std::mutex> lk(p->mu);
     auto it = p->group.find(dev);
     if (it == p->group.end()) {
@@ -141,12 +149,10 @@ bool group_shape(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &d
         it = p->group.emplace(dev, r).first;
     }
     GroupShape &r = *it->second;
-    // Time in rounds of tiles over the SMs, one tile at a time on each.
-    auto time = [&](int64_t n, double clk) {
-        return (alone ? (double)((n + sms - 1) / sms) : (double)n / sms) * (p->nchan * clk + kTileClocks);
-    };
-    while (!r.sizes.empty() && time(group_tiles(r, nsamp_out), r.sizes[0].clk) <=
-                                   kGain * time(tiles, direct_clocks(r.spread))) {
+    const double n = (double)group_tiles(r, nsamp_out) / sms;
+    while (!r.sizes.empty() &&
+           (alone ? std::ceil(n) : n) * (p->nchan * r.sizes[0].clk + kTileClocks) / kClocksPerUs <=
+               kGain * spread_factor(r.spread) * direct) {
         if (!r.entries) {
             GroupPrep a;
             a.dmshift = dt.dmshift;

@@ -116,7 +116,9 @@ struct dd_plan_s {
     bool tiles_auto[3] = {true, true, true};  // resolved by the plan until set
     std::mutex mu;
     std::map<int, dd::DevTables> dev;      // per CUDA device
+    bool tiles_open[3] = {true, true, true};  // executions may choose, until set
     std::map<uint64_t, dd::Geometry> geo;  // per (dtype, tiles) key
+    uint32_t shape_unfit[3] = {0, 0, 0};   // shapes found not to fit, a bit each
     // Remainder-DM launch per (dtype, tiles) key: (found, geometry).
     std::map<uint64_t, std::pair<bool, dd::Geometry>> tail_geo;
     std::map<int, std::shared_ptr<dd::GroupShape>> group;  // grouped execution, per device
@@ -162,6 +164,18 @@ dd_status make_geometry_range(dd_plan_s *p, dd_dtype t, const dd_tiles &tl, int 
 
 // Geometry for the plan's current tile shape, cached.
 dd_status plan_geometry(dd_plan_s *p, dd_dtype t, Geometry *g);
+
+// Geometry for one execution of nsamp_out samples: the plan's shape if the
+// caller or the autotuner set one, else the shape expected to finish first.
+dd_status execution_geometry(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, Geometry *g);
+
+// Neither the caller nor the autotuner has set the plan's shape.
+bool tiles_open(dd_plan_s *p, dd_dtype t);
+
+// Modelled time of the direct kernel in one of the shapes that
+// execution_geometry chooses from (-1 for another shape).
+double direct_time_us(dd_dtype t, const dd_tiles &tl, int nchan, int ndm, int64_t nsamp_out,
+                      int sms);
 
 // Launch shape for the DMs of the last, partly filled DM tile of geometry g,
 // run as a launch of their own (see dd_plan.cpp); cached per tile shape.

@@ -109,7 +109,7 @@ extern "C" dd_status dd_execute_noalloc(dd_plan_t p, const void *in, dd_dtype dt
                         std::to_string(kNoAllocBytes) + "-byte array; use dd_execute");
 
     dd::Geometry g;
-    if ((st = dd::plan_geometry(p, dtype, &g)) != DD_OK)
+    if ((st = dd::execution_geometry(p, dtype, nsamp_out, &g)) != DD_OK)
         return st;
     void *base = nullptr;
     if ((st = noalloc_base(&base)) != DD_OK)

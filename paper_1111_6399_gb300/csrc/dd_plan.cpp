@@ -54,9 +54,105 @@ void count_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 dd_tiles default_tiles(dd_dtype t) {
     switch (t) {
     case DD_U8:  return dd_tiles{4, 12, 1, 8, 8};
-    case DD_F16: return dd_tiles{1, 12, 1, 16, 8};
-    default:     return dd_tiles{2, 12, 1, 16, 8};
+    case DD_F16: return dd_tiles{4, 12, 1, 12, 8};
+    default:     return dd_tiles{4, 12, 1, 16, 8};
     }
+}
+
+namespace {
+
+// Tile shapes an execution chooses from, with the time of one round of tiles
+// (one CTA per SM, or `resident`) at 64 and 512 channels in microseconds:
+// each shape run for 8 rounds on a 300 MHz band at 1.5 GHz with unit DM
+// steps.  Large beams take the shape of the least time per output (the
+// preferred one, or one DM column more where that saves a round); small ones
+// a shape whose tiles are all resident at once.  With the preferred shape
+// alone, 64 channels x 64 DMs x 8192 samples took 29 us (16 CTAs on 152 SMs)
+// against 15, and 512 x 200 x 8192 took 153 against 71.
+struct ShapeCost {
+    dd_tiles tiles;
+    int resident;
+    double us64, us512;
+};
+const std::vector<ShapeCost> &shape_costs(dd_dtype t) {
+    static const std::vector<ShapeCost> u8 = {
+        {{4, 12, 1, 8, 8}, 1, 25.2, 155.0},  {{4, 13, 1, 8, 8}, 1, 26.8, 163.7},
+        {{4, 10, 1, 8, 8}, 1, 24.6, 148.9},  {{4, 8, 1, 8, 8}, 1, 21.1, 118.8},
+        {{2, 16, 1, 8, 8}, 1, 19.3, 110.0},  {{2, 13, 1, 8, 8}, 1, 17.3, 98.0},
+        {{2, 8, 1, 12, 8}, 1, 15.0, 76.4},   {{4, 8, 1, 16, 4}, 1, 14.8, 72.8},
+        {{2, 16, 1, 16, 4}, 1, 14.3, 75.1},  {{2, 13, 1, 16, 4}, 1, 12.8, 66.3},
+        {{2, 8, 1, 16, 4}, 1, 11.8, 60.4},   {{1, 8, 1, 16, 4}, 1, 10.8, 58.0}};
+    static const std::vector<ShapeCost> f16 = {
+        {{4, 12, 1, 12, 8}, 1, 24.0, 133.0}, {{4, 10, 1, 12, 8}, 1, 23.5, 127.0},
+        {{4, 8, 1, 12, 8}, 1, 19.3, 100.6},  {{2, 8, 1, 16, 8}, 1, 13.9, 75.6},
+        {{4, 8, 1, 16, 4}, 1, 13.8, 72.4},   {{2, 16, 1, 16, 4}, 1, 13.8, 80.9},
+        {{2, 8, 1, 16, 4}, 1, 11.2, 64.6},   {{1, 8, 1, 16, 4}, 2, 11.5, 69.0}};
+    static const std::vector<ShapeCost> f32 = {
+        {{4, 12, 1, 16, 8}, 1, 18.6, 113.4}, {{4, 6, 2, 16, 8}, 1, 18.4, 112.7},
+        {{4, 13, 1, 12, 8}, 1, 23.0, 128.8}, {{4, 10, 1, 16, 8}, 1, 16.2, 95.5},
+        {{4, 8, 1, 16, 8}, 1, 14.5, 81.6},   {{2, 16, 1, 16, 8}, 1, 14.0, 85.8},
+        {{2, 8, 1, 16, 8}, 1, 10.5, 61.5},   {{2, 8, 1, 24, 4}, 1, 9.2, 52.0},
+        {{1, 8, 1, 24, 4}, 2, 9.8, 54.0}};
+    return t == DD_U8 ? u8 : t == DD_F16 ? f16 : f32;
+}
+
+}  // namespace
+
+double direct_time_us(dd_dtype t, const dd_tiles &tl, int nchan, int ndm, int64_t nsamp_out,
+                      int sms) {
+    for (const ShapeCost &c : shape_costs(t)) {
+        if (std::memcmp(&c.tiles, &tl, sizeof(tl)) != 0)
+            continue;
+        const int64_t d = tl.dm_per_thread * tl.dm_warps;
+        const int64_t len = (int64_t)warp_span(t, tl.words_per_thread) * tl.time_warps;
+        const int64_t n = (ndm + d - 1) / d * ((nsamp_out + len - 1) / len);
+        const int64_t slots = (int64_t)sms * c.resident;
+        return (double)((n + slots - 1) / slots) *
+               std::max(0.5 * c.us64, c.us64 + (c.us512 - c.us64) * (nchan - 64) / 448.0);
+    }
+    return -1.0;
+}
+
+bool tiles_open(dd_plan_s *p, dd_dtype t) {
+    std::lock_guard<std::mutex> lk(p->mu);
+    return p->tiles_open[t];
+}
+
+dd_status execution_geometry(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, Geometry *g) {
+    int dev = 0;
+    int sms = 0;
+    if (valid_dtype(t) && cudaGetDevice(&dev) == cudaSuccess && (sms = sm_count(dev)) > 0) {
+        const std::vector<ShapeCost> &shapes = shape_costs(t);
+        std::lock_guard<std::mutex> lk(p->mu);
+        while (p->tiles_open[t]) {
+            int best = -1;
+            double best_us = 0;
+            for (int i = 0; i < (int)shapes.size(); ++i) {
+                if (p->shape_unfit[t] >> i & 1u)
+                    continue;
+                const double us =
+                    direct_time_us(t, shapes[i].tiles, p->nchan, p->ndm, nsamp_out, sms);
+                if (best < 0 || us < best_us) {
+                    best = i;
+                    best_us = us;
+                }
+            }
+            if (best < 0)
+                break;
+            const uint64_t key = geo_key(t, shapes[best].tiles);
+            auto it = p->geo.find(key);
+            Geometry r;
+            if (it == p->geo.end() && make_geometry(p, t, shapes[best].tiles, &r) == DD_OK)
+                it = p->geo.emplace(key, r).first;
+            if (it != p->geo.end()) {
+                *g = it->second;
+                return DD_OK;
+            }
+            // Its windows do not fit shared memory: passed over from now on.
+            p->shape_unfit[t] |= 1u << best;
+        }
+    }
+    return plan_geometry(p, t, g);
 }
 
 std::vector<dd_tiles> auto_tiles(dd_dtype t) {
@@ -69,7 +165,7 @@ std::vector<dd_tiles> auto_tiles(dd_dtype t) {
         const int nw = base.words_per_thread;
         const int wt = std::max(1, std::min(max_consumer_warps(dthr, nw) / wd,
                                             max_t_cta / warp_span(t, nw)));
-        for (int cs = base.chan_per_stage; cs >= 4; cs /= 2)
+        for (int cs = base.chan_per_stage; cs >= 4; cs = (cs / 2) & ~3)
             out.push_back(dd_tiles{dthr, wd, wt, cs, nw});
     }
     return out;
@@ -412,6 +508,7 @@ dd_status dd_plan_set_tiles(dd_plan_t p, dd_dtype t, const dd_tiles *tl) {
     std::lock_guard<std::mutex> lk(p->mu);
     p->tiles[t] = *tl;
     p->tiles_auto[t] = false;
+    p->tiles_open[t] = false;
     return DD_OK;
 }
 
