@@ -169,6 +169,10 @@ dd_status plan_geometry(dd_plan_s *p, dd_dtype t, Geometry *g);
 // caller or the autotuner set one, else the shape expected to finish first.
 dd_status execution_geometry(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, Geometry *g);
 
+// Modelled time of an execution by the direct kernel, to compare lengths by
+// (microseconds, or rounds of tiles where the shape has been set).
+double execution_time(dd_plan_s *p, dd_dtype t, int64_t nsamp_out);
+
 // Neither the caller nor the autotuner has set the plan's shape.
 bool tiles_open(dd_plan_s *p, dd_dtype t);
 

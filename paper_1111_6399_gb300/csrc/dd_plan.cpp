@@ -96,20 +96,23 @@ const std::vector<ShapeCost> &shape_costs(dd_dtype t) {
     return t == DD_U8 ? u8 : t == DD_F16 ? f16 : f32;
 }
 
+double shape_time_us(dd_dtype t, const ShapeCost &c, int nchan, int ndm, int64_t nsamp_out,
+                     int sms) {
+    const int64_t d = c.tiles.dm_per_thread * c.tiles.dm_warps;
+    const int64_t len = (int64_t)warp_span(t, c.tiles.words_per_thread) * c.tiles.time_warps;
+    const int64_t n = (ndm + d - 1) / d * ((nsamp_out + len - 1) / len);
+    const int64_t slots = (int64_t)sms * c.resident;
+    return (double)((n + slots - 1) / slots) *
+           std::max(0.5 * c.us64, c.us64 + (c.us512 - c.us64) * (nchan - 64) / 448.0);
+}
+
 }  // namespace
 
 double direct_time_us(dd_dtype t, const dd_tiles &tl, int nchan, int ndm, int64_t nsamp_out,
                       int sms) {
-    for (const ShapeCost &c : shape_costs(t)) {
-        if (std::memcmp(&c.tiles, &tl, sizeof(tl)) != 0)
-            continue;
-        const int64_t d = tl.dm_per_thread * tl.dm_warps;
-        const int64_t len = (int64_t)warp_span(t, tl.words_per_thread) * tl.time_warps;
-        const int64_t n = (ndm + d - 1) / d * ((nsamp_out + len - 1) / len);
-        const int64_t slots = (int64_t)sms * c.resident;
-        return (double)((n + slots - 1) / slots) *
-               std::max(0.5 * c.us64, c.us64 + (c.us512 - c.us64) * (nchan - 64) / 448.0);
-    }
+    for (const ShapeCost &c : shape_costs(t))
+        if (std::memcmp(&c.tiles, &tl, sizeof(tl)) == 0)
+            return shape_time_us(t, c, nchan, ndm, nsamp_out, sms);
     return -1.0;
 }
 
@@ -118,31 +121,41 @@ bool tiles_open(dd_plan_s *p, dd_dtype t) {
     return p->tiles_open[t];
 }
 
+namespace {
+
+// The listed shape expected to finish first (-1: none fits), and its time.
+int fastest_shape(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, int sms, double *us) {
+    const std::vector<ShapeCost> &shapes = shape_costs(t);
+    int best = -1;
+    for (int i = 0; i < (int)shapes.size(); ++i) {
+        if (p->shape_unfit[t] >> i & 1u)
+            continue;
+        const double u = shape_time_us(t, shapes[i], p->nchan, p->ndm, nsamp_out, sms);
+        if (best < 0 || u < *us) {
+            best = i;
+            *us = u;
+        }
+    }
+    return best;
+}
+
+}  // namespace
+
 dd_status execution_geometry(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, Geometry *g) {
     int dev = 0;
     int sms = 0;
     if (valid_dtype(t) && cudaGetDevice(&dev) == cudaSuccess && (sms = sm_count(dev)) > 0) {
-        const std::vector<ShapeCost> &shapes = shape_costs(t);
         std::lock_guard<std::mutex> lk(p->mu);
         while (p->tiles_open[t]) {
-            int best = -1;
-            double best_us = 0;
-            for (int i = 0; i < (int)shapes.size(); ++i) {
-                if (p->shape_unfit[t] >> i & 1u)
-                    continue;
-                const double us =
-                    direct_time_us(t, shapes[i].tiles, p->nchan, p->ndm, nsamp_out, sms);
-                if (best < 0 || us < best_us) {
-                    best = i;
-                    best_us = us;
-                }
-            }
+            double us = 0;
+            const int best = fastest_shape(p, t, nsamp_out, sms, &us);
             if (best < 0)
                 break;
-            const uint64_t key = geo_key(t, shapes[best].tiles);
+            const dd_tiles &tiles = shape_costs(t)[(size_t)best].tiles;
+            const uint64_t key = geo_key(t, tiles);
             auto it = p->geo.find(key);
             Geometry r;
-            if (it == p->geo.end() && make_geometry(p, t, shapes[best].tiles, &r) == DD_OK)
+            if (it == p->geo.end() && make_geometry(p, t, tiles, &r) == DD_OK)
                 it = p->geo.emplace(key, r).first;
             if (it != p->geo.end()) {
                 *g = it->second;
@@ -153,6 +166,22 @@ dd_status execution_geometry(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, Geomet
         }
     }
     return plan_geometry(p, t, g);
+}
+
+double execution_time(dd_plan_s *p, dd_dtype t, int64_t nsamp_out) {
+    int dev = 0;
+    const int sms = cudaGetDevice(&dev) == cudaSuccess ? std::max(1, sm_count(dev)) : 1;
+    {
+        std::lock_guard<std::mutex> lk(p->mu);
+        double us = 0;
+        if (p->tiles_open[t] && fastest_shape(p, t, nsamp_out, sms, &us) >= 0)
+            return us;
+    }
+    Geometry g;
+    if (plan_geometry(p, t, &g) != DD_OK)
+        return 1.0;
+    const int64_t n = (int64_t)g.ntile_d * ((nsamp_out + g.t_cta - 1) / g.t_cta);
+    return (double)((n + sms - 1) / sms);
 }
 
 std::vector<dd_tiles> auto_tiles(dd_dtype t) {
