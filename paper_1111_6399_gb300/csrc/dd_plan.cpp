@@ -77,16 +77,16 @@ struct ShapeCost {
 const std::vector<ShapeCost> &shape_costs(dd_dtype t) {
     static const std::vector<ShapeCost> u8 = {
         {{4, 12, 1, 8, 8}, 1, 25.2, 155.0},  {{4, 13, 1, 8, 8}, 1, 26.8, 163.7},
-        {{4, 10, 1, 8, 8}, 1, 24.6, 148.9},  {{4, 8, 1, 8, 8}, 1, 21.1, 118.8},
-        {{2, 16, 1, 8, 8}, 1, 19.3, 110.0},  {{2, 13, 1, 8, 8}, 1, 17.3, 98.0},
-        {{2, 8, 1, 12, 8}, 1, 15.0, 76.4},   {{4, 8, 1, 16, 4}, 1, 14.8, 72.8},
-        {{2, 16, 1, 16, 4}, 1, 14.3, 75.1},  {{2, 13, 1, 16, 4}, 1, 12.8, 66.3},
-        {{2, 8, 1, 16, 4}, 1, 11.8, 60.4},   {{1, 8, 1, 16, 4}, 1, 10.8, 58.0}};
+        {{4, 8, 1, 8, 8}, 1, 21.1, 118.8},   {{2, 16, 1, 8, 8}, 1, 19.3, 110.0},
+        {{2, 13, 1, 8, 8}, 1, 17.3, 98.0},   {{2, 8, 1, 12, 8}, 1, 15.0, 76.4},
+        {{4, 8, 1, 16, 4}, 1, 14.8, 72.8},   {{2, 16, 1, 16, 4}, 1, 14.3, 75.1},
+        {{2, 13, 1, 16, 4}, 1, 12.8, 66.3},  {{2, 8, 1, 16, 4}, 1, 11.8, 60.4},
+        {{1, 8, 1, 16, 4}, 1, 10.8, 58.0}};
     static const std::vector<ShapeCost> f16 = {
-        {{4, 12, 1, 12, 8}, 1, 24.0, 133.0}, {{4, 10, 1, 12, 8}, 1, 23.5, 127.0},
-        {{4, 8, 1, 12, 8}, 1, 19.3, 100.6},  {{2, 8, 1, 16, 8}, 1, 13.9, 75.6},
-        {{4, 8, 1, 16, 4}, 1, 13.8, 72.4},   {{2, 16, 1, 16, 4}, 1, 13.8, 80.9},
-        {{2, 8, 1, 16, 4}, 1, 11.2, 64.6},   {{1, 8, 1, 16, 4}, 2, 11.5, 69.0}};
+        {{4, 12, 1, 12, 8}, 1, 24.0, 133.0}, {{4, 8, 1, 12, 8}, 1, 19.3, 100.6},
+        {{2, 8, 1, 16, 8}, 1, 13.9, 75.6},   {{4, 8, 1, 16, 4}, 1, 13.8, 72.4},
+        {{2, 16, 1, 16, 4}, 1, 13.8, 80.9},  {{2, 8, 1, 16, 4}, 1, 11.2, 64.6},
+        {{1, 8, 1, 16, 4}, 2, 11.5, 69.0}};
     static const std::vector<ShapeCost> f32 = {
         {{4, 12, 1, 16, 8}, 1, 18.6, 113.4}, {{4, 6, 2, 16, 8}, 1, 18.4, 112.7},
         {{4, 13, 1, 12, 8}, 1, 23.0, 128.8}, {{4, 10, 1, 16, 8}, 1, 16.2, 95.5},
