@@ -16,22 +16,21 @@
 //
 // Main path, fused_kernel: one thread-block cluster per channel, its cs CTAs
 // (1, 2, 4 or 8) each owning m consecutive output samples.  A CTA streams its
-// voltages once (each warp reads 32 samples' bytes in 512-byte coalesced
-// steps, the 16-byte words of one sample summed over neighbouring lanes),
-// keeps P in shared memory, and every clipping pass sums its own P; the
-// cluster's partial sums meet in rank 0's shared memory (distributed shared
-// memory, hardware cluster barriers), rank 0 derives the statistics and the
-// others read them back.  HBM traffic is the compulsory minimum: 4*nint bytes
+// voltages once (each warp reads 32 samples' bytes in coalesced steps, the
+// words of one sample summed over neighbouring lanes), keeps P in shared
+// memory, and every clipping pass sums its own P; each CTA reads the partial
+// sums of its cluster (distributed shared memory, hardware cluster barriers)
+// and derives the statistics.  HBM traffic is the compulsory minimum: 4*nint bytes
 // of voltages per output sample in, 1 byte of code out.
 //
 // Fallback for rows whose P does not fit a cluster's shared memory: P in the
-// caller's work array and niter + 1 launches -- power_kernel (one thread per
-// output sample; P and pass 1's sums), clip_kernel for passes 2..niter and
+// caller's work array and niter + 1 launches -- power_kernel (P and pass 1's sums), clip_kernel for passes 2..niter and
 // quantize_kernel, each block deriving its channel's statistics from the
 // exact sums itself.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <string>
 
@@ -40,6 +39,7 @@
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int64_t kFallbackBlocks = 152 * 8 * 4;
 
 struct Acc {  // exact per-channel sums of one clipping pass
     unsigned long long cnt, s1, s2;
@@ -67,8 +67,8 @@ __device__ __forceinline__ Stats stats_of(const Acc &a, double k) {
     return s;
 }
 
-// Block sums of (cnt, s1, s2), then one atomic triple per block.  P <= 2^22,
-// so a block's P^2 sum stays below 2^62.
+// Block sums of (cnt, s1, s2), then one atomic triple per block.  P <= 2^22 and
+// a row has at most 2^19 samples, so the P^2 sum stays below 2^64.
 __device__ __forceinline__ void block_accumulate(unsigned long long cnt, unsigned long long s1,
                                                  unsigned long long s2, Acc *dst) {
     __shared__ unsigned long long red[3][kThreads / 32];
@@ -106,10 +106,12 @@ __global__ void __launch_bounds__(kThreads) power_kernel(const uint8_t *__restri
                                                          int nint, uint32_t *__restrict__ p_out,
                                                          Acc *acc) {
     const int c = blockIdx.y;
-    const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    uint32_t p = 0;
-    if (t < n) {
+    unsigned long long cnt = 0, s1 = 0, s2 = 0;
+    const int64_t step = (int64_t)gridDim.x * kThreads;
+#pragma unroll 4
+    for (int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x; t < n; t += step) {
         const uint8_t *src = volts + (int64_t)c * pitch + 4 * t * nint;
+        uint32_t p = 0;
         if (VEC) {
             for (int j = 0; j < nint; j += 4) {
                 const uint4 v = *reinterpret_cast<const uint4 *>(src + 4 * j);
@@ -123,8 +125,11 @@ __global__ void __launch_bounds__(kThreads) power_kernel(const uint8_t *__restri
             }
         }
         p_out[(int64_t)c * prow + t] = p;
+        cnt += 1;
+        s1 += p;
+        s2 += (unsigned long long)p * p;
     }
-    block_accumulate(t < n ? 1ull : 0ull, p, (unsigned long long)p * p, &acc[c]);
+    block_accumulate(cnt, s1, s2, &acc[c]);
 }
 
 // One clipping pass: sums over the samples at or below the previous pass's
@@ -138,9 +143,10 @@ __global__ void __launch_bounds__(kThreads) clip_kernel(const uint32_t *__restri
         sthr = stats_of(prev[c], k).thr;
     __syncthreads();
     const long long thr = sthr;
-    const int64_t t = 4 * ((int64_t)blockIdx.x * kThreads + threadIdx.x);
+    const int64_t step = 4 * (int64_t)gridDim.x * kThreads;
     unsigned long long cnt = 0, s1 = 0, s2 = 0;
-    if (t < n) {
+#pragma unroll 4
+    for (int64_t t = 4 * ((int64_t)blockIdx.x * kThreads + threadIdx.x); t < n; t += step) {
         const uint4 q = *reinterpret_cast<const uint4 *>(p_in + (int64_t)c * prow + t);
         const uint32_t v[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
@@ -155,14 +161,25 @@ __global__ void __launch_bounds__(kThreads) clip_kernel(const uint32_t *__restri
     block_accumulate(cnt, s1, s2, &next[c]);
 }
 
-__device__ __forceinline__ uint32_t code_of(uint32_t p, long long thr, float m, float s,
-                                            bool flat) {
-    if (flat || (long long)p > thr)
-        return 128u;
-    const float d = __fsub_rn(__uint2float_rn(p), m);
-    float v = rintf(__fadd_rn(128.0f, __fmul_rn(d, s)));
-    v = v < 0.0f ? 0.0f : (v > 255.0f ? 255.0f : v);
-    return (uint32_t)v;
+// Threshold as a 32-bit value (P is at most 2^22): -1 keeps nothing.
+__device__ __forceinline__ int thr32(long long thr) {
+    return thr < 0 ? -1 : thr > 0x7fffffff ? 0x7fffffff : (int)thr;
+}
+
+// p + 2^23 (exact) less 2^23 is (float)p, and v + 2^23 rounds v in [0, 255] to
+// the nearest integer, ties to even, in its low byte: conversions and rintf
+// would go through a unit of a quarter of the rate.  A NaN gives code 0.
+__device__ __forceinline__ uint32_t code_of(uint32_t p, int thr, float m, float s, bool flat) {
+    const float f = __fsub_rn(__uint_as_float(p | 0x4b000000u), 8388608.0f);
+    const float v = __fadd_rn(128.0f, __fmul_rn(__fsub_rn(f, m), s));
+    const uint32_t q =
+        __float_as_uint(__fadd_rn(fminf(fmaxf(v, 0.0f), 255.0f), 8388608.0f)) & 255u;
+    return flat || (int)p > thr ? 128u : q;
+}
+
+__device__ __forceinline__ uint32_t codes_of(uint4 p, int thr, float m, float s, bool flat) {
+    return code_of(p.x, thr, m, s, flat) | code_of(p.y, thr, m, s, flat) << 8 |
+           code_of(p.z, thr, m, s, flat) << 16 | code_of(p.w, thr, m, s, flat) << 24;
 }
 
 __global__ void __launch_bounds__(kThreads) quantize_kernel(const uint32_t *__restrict__ p_in,
@@ -187,21 +204,20 @@ __global__ void __launch_bounds__(kThreads) quantize_kernel(const uint32_t *__re
     }
     __syncthreads();
     const float m = sm, s = ss;
-    const long long thr = sthr;
+    const int thr = thr32(sthr);
     const bool flat = sflat != 0;
-    const int64_t t = 4 * ((int64_t)blockIdx.x * kThreads + threadIdx.x);
-    if (t >= n)
-        return;
-    const uint4 q = *reinterpret_cast<const uint4 *>(p_in + (int64_t)c * prow + t);
-    uint8_t *dst = out + (int64_t)c * out_pitch + t;
-    if (t + 4 <= n) {
-        *reinterpret_cast<uint32_t *>(dst) =
-            code_of(q.x, thr, m, s, flat) | code_of(q.y, thr, m, s, flat) << 8 |
-            code_of(q.z, thr, m, s, flat) << 16 | code_of(q.w, thr, m, s, flat) << 24;
-    } else {
-        const uint32_t v[4] = {q.x, q.y, q.z, q.w};
-        for (int i = 0; t + i < n; ++i)
-            dst[i] = (uint8_t)code_of(v[i], thr, m, s, flat);
+    const int64_t step = 4 * (int64_t)gridDim.x * kThreads;
+#pragma unroll 4
+    for (int64_t t = 4 * ((int64_t)blockIdx.x * kThreads + threadIdx.x); t < n; t += step) {
+        const uint4 q = *reinterpret_cast<const uint4 *>(p_in + (int64_t)c * prow + t);
+        uint8_t *dst = out + (int64_t)c * out_pitch + t;
+        if (t + 4 <= n) {
+            *reinterpret_cast<uint32_t *>(dst) = codes_of(q, thr, m, s, flat);
+        } else {
+            const uint32_t v[4] = {q.x, q.y, q.z, q.w};
+            for (int i = 0; t + i < n; ++i)
+                dst[i] = (uint8_t)code_of(v[i], thr, m, s, flat);
+        }
     }
 }
 
@@ -216,10 +232,9 @@ constexpr int64_t kFusedSmemMax = 200 * 1024;     // P bytes per CTA allowed
 constexpr int kMaxCluster = 8;
 
 struct Params {
-    long long thr;
+    int thr;
     float m, s;
     int flat;
-    double mean, sd;
 };
 
 // Block sums of (cnt, s1, s2) for kFusedThreads threads, left in red[][0] for
@@ -251,15 +266,43 @@ __device__ __forceinline__ void fused_block_sum(unsigned long long v[3],
 }
 
 __device__ __forceinline__ uint32_t fused_power_word(uint4 v) {
-    return (uint32_t)(__dp4a((int)v.x, (int)v.x, 0) + __dp4a((int)v.y, (int)v.y, 0) +
-                      __dp4a((int)v.z, (int)v.z, 0) + __dp4a((int)v.w, (int)v.w, 0));
+    return (uint32_t)__dp4a((int)v.x, (int)v.x,
+                            __dp4a((int)v.y, (int)v.y,
+                                   __dp4a((int)v.z, (int)v.z, __dp4a((int)v.w, (int)v.w, 0))));
 }
 
-// Q = nint/4 16-byte words per output sample (1..16); Q = 0: 4-byte loads,
-// one thread per sample (nint < 4 or rows not 16-byte aligned).
+// Values i of the Q lanes of a group summed over the group; lane l leaves with
+// value l % Q (Q - 1 shuffles for Q sums).
 template <int Q>
-__global__ void __launch_bounds__(kFusedThreads) fused_kernel(
-    const uint8_t *__restrict__ volts, int64_t pitch, int64_t n, int nint, int m, double k,
+__device__ __forceinline__ uint32_t reduce_scatter(uint32_t (&a)[Q], int lane) {
+#pragma unroll
+    for (int h = Q / 2; h > 0; h >>= 1) {
+        const bool upper = (lane & h) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const uint32_t keep = upper ? a[i + h] : a[i], send = upper ? a[i] : a[i + h];
+            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+        }
+    }
+    return a[0];
+}
+
+// NINT raw samples per output sample; V16: rows on 16 bytes.
+//
+// HBM-bound at 16 raw samples per output as far as the passes over P overlap
+// the other CTA's loads, so those are kept short: 16-byte reads of P, 32-bit
+// counts and sums (a thread has at most 100 values of 2^22), codes without
+// conversion instructions, and one cluster barrier per pass (every CTA reads
+// all partial sums and derives the statistics itself).  256 channels x
+// 2362048 raw samples, nint 16, 3 passes: 436 us (363 us of HBM traffic; 450
+// with scalar reads and 64-bit sums); 200 x 1048576, nint 64, 5 passes: 145
+// (222).  Loads are whole warps of consecutive words, and the words of an
+// output sample meet by a reduce-scatter, one output per lane: 77 x 51434,
+// nint 32, rows off 16 bytes: 8.7 us (31 with a thread per output); nint 1,
+// 135 x 183608: 84 (196).
+template <int NINT, bool V16>
+__global__ void __launch_bounds__(kFusedThreads, 2) fused_kernel(
+    const uint8_t *__restrict__ volts, int64_t pitch, int64_t n, int m, double k,
     int niter, uint8_t *__restrict__ out, int64_t out_pitch, double *mean_out, double *sd_out) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
@@ -269,7 +312,7 @@ __global__ void __launch_bounds__(kFusedThreads) fused_kernel(
     extern __shared__ uint4 fused_smem[];
     uint32_t *P = reinterpret_cast<uint32_t *>(fused_smem);
     __shared__ unsigned long long red[3][kFusedWarps];
-    __shared__ unsigned long long part[3];
+    __shared__ unsigned long long part[2][3];  // of even and odd passes
     __shared__ Params prm;
 
     const int64_t t0 = (int64_t)rank * m;
@@ -278,117 +321,225 @@ __global__ void __launch_bounds__(kFusedThreads) fused_kernel(
     unsigned long long acc[3] = {0, 0, 0};
 
     // Pass 1: P = integrated Stokes I, kept in shared memory.
-    if (Q > 0) {
-        constexpr int QD = Q > 0 ? Q : 1;  // Q, without a zero divisor in the Q = 0 body
-        const uint4 *row = reinterpret_cast<const uint4 *>(volts + (int64_t)c * pitch) + t0 * QD;
-        constexpr int U = QD >= 8 ? 1 : 2;  // groups of 32 samples in flight per warp
+    if constexpr (V16 && NINT >= 4) {
+        constexpr int Q = NINT / 4;  // 16-byte words per output sample
+        const uint4 *row = reinterpret_cast<const uint4 *>(volts + (int64_t)c * pitch) + t0 * Q;
+        constexpr int U = Q >= 8 ? 1 : 8 / Q;  // groups of 32 samples in flight per warp
+        constexpr int L = Q > 8 ? 8 : Q;       // words of a group in flight
         for (int g0 = warp * 32; g0 < len; g0 += kFusedWarps * 32 * U) {
-            uint4 v[U][QD];
+            uint32_t a[U][Q];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int g = g0 + u * kFusedWarps * 32;
+            for (int j0 = 0; j0 < Q; j0 += L) {
+                uint4 v[U][L];
 #pragma unroll
-                for (int j = 0; j < QD; ++j) {
-                    const int ci = lane + 32 * j;
-                    if (g + ci / QD < len)
-                        v[u][j] = __ldcs(row + (int64_t)g * QD + ci);
-                    else
-                        v[u][j] = make_uint4(0, 0, 0, 0);
-                }
-            }
+                for (int u = 0; u < U; ++u) {
+                    const int g = g0 + u * kFusedWarps * 32;
+                    const uint4 *src = row + (int64_t)g * Q + lane + 32 * j0;
+                    if (g + 32 <= len) {
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int g = g0 + u * kFusedWarps * 32;
+                        for (int j = 0; j < L; ++j)
+                            v[u][j] = __ldcs(src + 32 * j);
+                    } else {
 #pragma unroll
-                for (int j = 0; j < QD; ++j) {
-                    uint32_t p = fused_power_word(v[u][j]);
-#pragma unroll
-                    for (int o = QD / 2; o > 0; o >>= 1)
-                        p += __shfl_xor_sync(0xffffffffu, p, o);
-                    const int sl = g + (32 * j + lane) / QD;
-                    if (lane % QD == 0 && sl < len) {
-                        P[sl] = p;
-                        acc[1] += p;
-                        acc[2] += (unsigned long long)p * p;
+                        for (int j = 0; j < L; ++j)
+                            v[u][j] = g + (lane + 32 * (j0 + j)) / Q < len ? __ldcs(src + 32 * j)
+                                                                           : make_uint4(0, 0, 0, 0);
                     }
                 }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int j = 0; j < L; ++j)
+                        a[u][j0 + j] = fused_power_word(v[u][j]);
             }
-        }
-    } else {
-        const uint8_t *row = volts + (int64_t)c * pitch + 4 * t0 * nint;
-        for (int sl = tid; sl < len; sl += kFusedThreads) {
-            const int *src = reinterpret_cast<const int *>(row + (int64_t)4 * nint * sl);
-            uint32_t p = 0;
-            for (int j = 0; j < nint; ++j) {
-                const int w = __ldcs(src + j);
-                p += (uint32_t)__dp4a(w, w, 0);
-            }
-            P[sl] = p;
-            acc[1] += p;
-            acc[2] += (unsigned long long)p * p;
-        }
-    }
-    acc[0] = tid == 0 ? (unsigned long long)len : 0ull;
-
-    long long thr = 0;
-    Params pr;
-    for (int it = 0; it < niter; ++it) {
-        if (it > 0) {
-            acc[0] = acc[1] = acc[2] = 0;
-            for (int sl = tid; sl < len; sl += kFusedThreads) {
-                const uint32_t p = P[sl];
-                if ((long long)p <= thr) {
-                    acc[0] += 1;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t p = reduce_scatter<Q>(a[u], lane);
+                const int sl = g0 + u * kFusedWarps * 32 + 32 / Q * (lane % Q) + lane / Q;
+                if (sl < len) {
+                    P[sl] = p;
                     acc[1] += p;
                     acc[2] += (unsigned long long)p * p;
                 }
             }
         }
-        fused_block_sum(acc, red);
-        if (tid == 0) {
-            part[0] = acc[0];
-            part[1] = acc[1];
-            part[2] = acc[2];
-        }
-        cluster.sync();  // every rank's part is written
-        if (rank == 0 && tid == 0) {
-            Acc a = {0, 0, 0};
-            for (unsigned q = 0; q < cs; ++q) {
-                const unsigned long long *rp = cluster.map_shared_rank(part, q);
-                a.cnt += rp[0];
-                a.s1 += rp[1];
-                a.s2 += rp[2];
+    } else if constexpr (V16) {
+        constexpr int W = 4 / NINT;  // output samples of a 16-byte word
+        const uint4 *row = reinterpret_cast<const uint4 *>(volts + (int64_t)c * pitch) + t0 / W;
+        constexpr int U = 4;
+        const int words = (len + W - 1) / W;
+        // A row may end within its last word: its samples one by one.
+        const int whole = len / W;
+        for (int w0 = tid; w0 < words; w0 += U * kFusedThreads) {
+            uint4 v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int w = w0 + u * kFusedThreads;
+                if (w < whole) {
+                    v[u] = __ldcs(row + w);
+                } else {
+                    const int *src = reinterpret_cast<const int *>(row + w);
+                    const int in = (len - w * W) * NINT;  // raw samples (< 4, or none)
+                    v[u].x = in > 0 ? (uint32_t)__ldcs(src) : 0u;
+                    v[u].y = in > 1 ? (uint32_t)__ldcs(src + 1) : 0u;
+                    v[u].z = in > 2 ? (uint32_t)__ldcs(src + 2) : 0u;
+                    v[u].w = 0u;
+                }
             }
-            const Stats st = stats_of(a, k);
-            prm.thr = st.thr;
-            prm.mean = st.mean;
-            prm.sd = st.sd;
-            prm.flat = st.sd > 0.0 ? 0 : 1;
-            prm.m = (float)st.mean;
-            prm.s = st.sd > 0.0 ? (float)__ddiv_rn(16.0, st.sd) : 0.0f;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int w = w0 + u * kFusedThreads;
+                if (w >= words)
+                    continue;
+                const uint32_t x[4] = {(uint32_t)__dp4a((int)v[u].x, (int)v[u].x, 0),
+                                       (uint32_t)__dp4a((int)v[u].y, (int)v[u].y, 0),
+                                       (uint32_t)__dp4a((int)v[u].z, (int)v[u].z, 0),
+                                       (uint32_t)__dp4a((int)v[u].w, (int)v[u].w, 0)};
+                // Samples past the end are 0: they add nothing (P is a whole
+                // number of words).
+                if constexpr (W == 4) {
+                    *reinterpret_cast<uint4 *>(P + 4 * w) = make_uint4(x[0], x[1], x[2], x[3]);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        acc[1] += x[i];
+                        acc[2] += (unsigned long long)x[i] * x[i];
+                    }
+                } else {
+                    const uint32_t p0 = x[0] + x[1], p1 = x[2] + x[3];
+                    *reinterpret_cast<uint2 *>(P + 2 * w) = make_uint2(p0, p1);
+                    acc[1] += p0;
+                    acc[1] += p1;
+                    acc[2] += (unsigned long long)p0 * p0;
+                    acc[2] += (unsigned long long)p1 * p1;
+                }
+            }
         }
-        cluster.sync();  // rank 0's prm is written; part may be reused after the next sum
-        pr = *cluster.map_shared_rank(&prm, 0);
-        thr = pr.thr;
+    } else {
+        // As for 16-byte words, with raw samples: lane l reads words l + 32 j.
+        const int *row =
+            reinterpret_cast<const int *>(volts + (int64_t)c * pitch) + t0 * NINT;
+        constexpr int A = NINT > 32 ? 32 : NINT;   // sums to scatter
+        constexpr int U = NINT >= 16 ? 1 : 16 / NINT;
+        constexpr int L = NINT > 16 ? 16 : NINT;   // loads of a group in flight
+        for (int g0 = warp * 32; g0 < len; g0 += kFusedWarps * 32 * U) {
+            uint32_t a[U][A];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int i = 0; i < A; ++i)
+                    a[u][i] = 0;
+#pragma unroll
+            for (int j0 = 0; j0 < NINT; j0 += L) {
+                int v[U][L];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int g = g0 + u * kFusedWarps * 32;
+                    const int *src = row + (int64_t)g * NINT + lane + 32 * j0;
+#pragma unroll
+                    for (int j = 0; j < L; ++j)
+                        v[u][j] = g + 32 <= len || g + (lane + 32 * (j0 + j)) / NINT < len
+                                      ? __ldcs(src + 32 * j)
+                                      : 0;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int j = 0; j < L; ++j)
+                        a[u][(j0 + j) / (NINT / A)] = (uint32_t)__dp4a(
+                            v[u][j], v[u][j], (int)a[u][(j0 + j) / (NINT / A)]);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t p = reduce_scatter<A>(a[u], lane);
+                const int sl = g0 + u * kFusedWarps * 32 + 32 / A * (lane % A) + lane / A;
+                if (sl < len) {
+                    P[sl] = p;
+                    acc[1] += p;
+                    acc[2] += (unsigned long long)p * p;
+                }
+            }
+        }
     }
-    // Rank 0 keeps its shared memory until every rank has read prm.
+    acc[0] = tid == 0 ? (unsigned long long)len : 0ull;
+
+    int thr = 0;
+    for (int it = 0; it < niter; ++it) {
+        if (it > 0) {
+            uint32_t cnt = 0, sum = 0;
+            unsigned long long sq = 0;
+            auto take = [&](uint32_t p) {
+                const bool kept = (int)p <= thr;
+                const uint32_t q = kept ? p : 0u;
+                cnt += kept ? 1u : 0u;
+                sum += q;
+                sq += (unsigned long long)q * q;
+            };
+            for (int sl = 4 * tid; sl < len; sl += 4 * kFusedThreads) {
+                if (sl + 4 <= len) {
+                    const uint4 p = *reinterpret_cast<const uint4 *>(P + sl);
+                    take(p.x);
+                    take(p.y);
+                    take(p.z);
+                    take(p.w);
+                } else {
+                    for (int i = sl; i < len; ++i)
+                        take(P[i]);
+                }
+            }
+            acc[0] = cnt;
+            acc[1] = sum;
+            acc[2] = sq;
+        }
+        fused_block_sum(acc, red);  // P is written, too, for every thread
+        if (tid == 0) {
+            part[it & 1][0] = acc[0];
+            part[it & 1][1] = acc[1];
+            part[it & 1][2] = acc[2];
+        }
+        cluster.sync();  // every rank's part is written, and that of two passes ago read
+        if (warp == 0) {
+            unsigned long long v[3] = {0, 0, 0};
+            if ((unsigned)lane < cs) {
+                const unsigned long long *rp = cluster.map_shared_rank(part[it & 1], lane);
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+                    v[i] = rp[i];
+            }
+#pragma unroll
+            for (int o = kMaxCluster / 2; o > 0; o >>= 1)
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+                    v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+            if (lane == 0) {
+                const Acc a = {v[0], v[1], v[2]};
+                const Stats st = stats_of(a, k);
+                prm.thr = thr32(st.thr);
+                if (it == niter - 1) {
+                    prm.flat = st.sd > 0.0 ? 0 : 1;
+                    prm.m = (float)st.mean;
+                    prm.s = st.sd > 0.0 ? (float)__ddiv_rn(16.0, st.sd) : 0.0f;
+                    if (rank == 0) {
+                        mean_out[c] = st.mean;
+                        sd_out[c] = st.sd;
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        thr = prm.thr;
+    }
+    // A CTA keeps its shared memory until every rank has read its part.
     asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
-    if (rank == 0 && tid == 0) {
-        mean_out[c] = pr.mean;
-        sd_out[c] = pr.sd;
-    }
-    const bool flat = pr.flat != 0;
+    const float mean = prm.m, scale = prm.s;
+    const bool flat = prm.flat != 0;
     uint8_t *dst = out + (int64_t)c * out_pitch + t0;
     for (int sl = 4 * tid; sl < len; sl += 4 * kFusedThreads) {
         if (sl + 4 <= len) {
             const uint4 q = *reinterpret_cast<const uint4 *>(P + sl);
-            *reinterpret_cast<uint32_t *>(dst + sl) =
-                code_of(q.x, thr, pr.m, pr.s, flat) | code_of(q.y, thr, pr.m, pr.s, flat) << 8 |
-                code_of(q.z, thr, pr.m, pr.s, flat) << 16 |
-                code_of(q.w, thr, pr.m, pr.s, flat) << 24;
+            *reinterpret_cast<uint32_t *>(dst + sl) = codes_of(q, thr, mean, scale, flat);
         } else {
             for (int i = sl; i < len; ++i)
-                dst[i] = (uint8_t)code_of(P[i], thr, pr.m, pr.s, flat);
+                dst[i] = (uint8_t)code_of(P[i], thr, mean, scale, flat);
         }
     }
     asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
@@ -398,9 +549,9 @@ __global__ void __launch_bounds__(kFusedThreads) fused_kernel(
 // first sample starts a warp group and a 4-byte output word).
 int64_t fused_m(int64_t n, int cs) { return ((n + cs - 1) / cs + 31) / 32 * 32; }
 
-template <int Q>
+template <int NINT, bool V16>
 cudaError_t launch_fused_q(int cs, int64_t m, const uint8_t *v, int64_t pitch, int64_t n,
-                           int nint, int nchan, double k, int niter, uint8_t *out,
+                           int nchan, double k, int niter, uint8_t *out,
                            int64_t out_pitch, double *mean, double *sd, cudaStream_t s,
                            bool *fits) {
     static unsigned long long attr_set = 0;  // per device
@@ -409,7 +560,7 @@ cudaError_t launch_fused_q(int cs, int64_t m, const uint8_t *v, int64_t pitch, i
     if (e != cudaSuccess)
         return e;
     if (dev >= 64 || !((attr_set >> dev) & 1ull)) {
-        e = cudaFuncSetAttribute(fused_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(fused_kernel<NINT, V16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kFusedSmemMax);
         if (e != cudaSuccess)
             return e;
@@ -429,14 +580,14 @@ cudaError_t launch_fused_q(int cs, int64_t m, const uint8_t *v, int64_t pitch, i
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int clusters = 0;
-    e = cudaOccupancyMaxActiveClusters(&clusters, fused_kernel<Q>, &cfg);
+    e = cudaOccupancyMaxActiveClusters(&clusters, fused_kernel<NINT, V16>, &cfg);
     if (e != cudaSuccess || clusters < 1) {
         (void)cudaGetLastError();  // not an error of the call: leave it to the fallback path
         *fits = false;
         return cudaSuccess;
     }
     *fits = true;
-    return cudaLaunchKernelEx(&cfg, fused_kernel<Q>, v, pitch, n, nint, (int)m, k, niter, out,
+    return cudaLaunchKernelEx(&cfg, fused_kernel<NINT, V16>, v, pitch, n, (int)m, k, niter, out,
                               out_pitch, mean, sd);
 }
 
@@ -491,26 +642,30 @@ extern "C" dd_status dd_frontend(const void *volts, int64_t volts_pitch, int nch
         return DD_OK;
     }
     const uint8_t *v = static_cast<const uint8_t *>(volts);
-    const bool vec = nint % 4 == 0 && ((uintptr_t)volts & 15u) == 0 && volts_pitch % 16 == 0;
+    const bool rows16 = ((uintptr_t)volts & 15u) == 0 && volts_pitch % 16 == 0;
+    const bool vec = nint % 4 == 0 && rows16;
     int cs = 1;
     while (cs < kMaxCluster && 4 * fused_m(n, cs) > kFusedSmemTarget)
         cs *= 2;
     if (4 * fused_m(n, cs) <= kFusedSmemMax) {
         const int64_t m = fused_m(n, cs);
         bool fits = false;
-        const int q = vec ? nint / 4 : 0;
-        switch (q) {
-#define DD_FE_CASE(QQ)                                                                       \
-    case QQ:                                                                                 \
-        e = launch_fused_q<QQ>(cs, m, v, volts_pitch, n, nint, nchan, k_clip, niter, out,     \
-                               out_pitch, mean, std_out, s, &fits);                          \
+        switch (nint) {
+#define DD_FE_CASE(NN)                                                                       \
+    case NN:                                                                                 \
+        e = rows16 ? launch_fused_q<NN, true>(cs, m, v, volts_pitch, n, nchan, k_clip, niter,\
+                                              out, out_pitch, mean, std_out, s, &fits)       \
+                   : launch_fused_q<NN, false>(cs, m, v, volts_pitch, n, nchan, k_clip,      \
+                                               niter, out, out_pitch, mean, std_out, s,      \
+                                               &fits);                                       \
         break;
-            DD_FE_CASE(0)
             DD_FE_CASE(1)
             DD_FE_CASE(2)
             DD_FE_CASE(4)
             DD_FE_CASE(8)
             DD_FE_CASE(16)
+            DD_FE_CASE(32)
+            DD_FE_CASE(64)
 #undef DD_FE_CASE
         default:
             return fail(DD_ERR_INVALID, "frontend: no kernel for this nint");
@@ -528,21 +683,29 @@ extern "C" dd_status dd_frontend(const void *volts, int64_t volts_pitch, int nch
     e = cudaMemsetAsync(acc, 0, sizeof(Acc) * niter * nchan, s);
     if (e != cudaSuccess)
         return fail(DD_ERR_CUDA, std::string("frontend memset: ") + cudaGetErrorString(e));
-    const dim3 g1((unsigned)((n + kThreads - 1) / kThreads), (unsigned)nchan);
+    // A block ends in three atomics on its channel's sums or begins with the
+    // statistics in FP64, so there are no more blocks than fill the device a
+    // few times (a block per 256 or 1024 samples took 2.3 ms for 300 channels
+    // x 524288 samples against 1.0 ms).
+    auto blocks = [&](int64_t per_block) {
+        return dim3((unsigned)std::min((n + per_block - 1) / per_block,
+                                       (int64_t)(kFallbackBlocks + nchan - 1) / nchan),
+                    (unsigned)nchan);
+    };
+    const dim3 g1 = blocks(kThreads), gc = blocks(4 * kThreads);
     // 16-byte loads need 16-byte aligned rows and whole groups of 4 samples.
     if (vec)
         power_kernel<true><<<g1, kThreads, 0, s>>>(v, volts_pitch, n, prow, nint, p, acc);
     else
         power_kernel<false><<<g1, kThreads, 0, s>>>(v, volts_pitch, n, prow, nint, p, acc);
     e = cudaGetLastError();
-    const dim3 g4((unsigned)((n + 4 * kThreads - 1) / (4 * kThreads)), (unsigned)nchan);
     for (int it = 1; it < niter && e == cudaSuccess; ++it) {
-        clip_kernel<<<g4, kThreads, 0, s>>>(p, n, prow, k_clip, acc + (int64_t)(it - 1) * nchan,
+        clip_kernel<<<gc, kThreads, 0, s>>>(p, n, prow, k_clip, acc + (int64_t)(it - 1) * nchan,
                                             acc + (int64_t)it * nchan);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
-        quantize_kernel<<<g4, kThreads, 0, s>>>(p, n, prow, k_clip,
+        quantize_kernel<<<gc, kThreads, 0, s>>>(p, n, prow, k_clip,
                                                 acc + (int64_t)(niter - 1) * nchan, out,
                                                 out_pitch, mean, std_out);
         e = cudaGetLastError();
