@@ -24,9 +24,9 @@
 // of voltages per output sample in, 1 byte of code out.
 //
 // Fallback for rows whose P does not fit a cluster's shared memory: P in the
-// caller's work array and niter + 1 launches -- power_kernel (P and pass 1's sums), clip_kernel for passes 2..niter and
-// quantize_kernel, each block deriving its channel's statistics from the
-// exact sums itself.
+// caller's work array and niter + 1 launches -- power_kernel (P and pass 1's
+// sums), clip_kernel for passes 2..niter and quantize_kernel, each block
+// deriving its channel's statistics from the exact sums itself.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
