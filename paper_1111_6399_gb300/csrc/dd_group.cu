@@ -374,10 +374,14 @@ __global__ void __launch_bounds__(kThreads, 1) group_kernel(const __grid_constan
 }
 
 // ---------------------------------------------------------------------------
-// The table: one thread per (DM tile, group), in two launches.
+// The table: one warp per (DM tile, group), in two launches.  A lane has two of
+// the tile's DMs, then one of the group's patterns (64 DMs and 24 patterns in
+// one thread took 120 us for a table of any size, against 12 us for 1 MB and 26 us
+// for 11 MB).
 // ---------------------------------------------------------------------------
 
-constexpr int kPrepThreads = 32;  // many small blocks: the threads are serial
+constexpr int kPrepThreads = 128;
+static_assert(kGroupDmCta == 64 && kGroupTuples <= 32, "two DMs, one pattern a lane");
 
 // Channels of one group: reference (smallest delay) first, so that every
 // delta_i is >= 0 (the shift rule is monotone in the delay).
@@ -425,7 +429,9 @@ __device__ uint32_t nibble(uint32_t key, int i) { return (key >> (4 * i)) & 15u;
 // Records and words of each group, as if its arrays came first; sizes: bytes
 // of its arrays.
 __global__ void __launch_bounds__(kPrepThreads) group_prep_kernel(const GroupPrep a, int *sizes) {
-    const int td = blockIdx.y, g = blockIdx.x * kPrepThreads + threadIdx.x;
+    constexpr uint32_t kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int td = blockIdx.y, g = (blockIdx.x * kPrepThreads + threadIdx.x) / 32;
     const int np = ((a.nchan + a.G - 1) / a.G + 1) / 2, ng = 2 * np;
     if (g >= ng)
         return;
@@ -433,56 +439,47 @@ __global__ void __launch_bounds__(kPrepThreads) group_prep_kernel(const GroupPre
     GroupEntry *tile = a.entries + (int64_t)td * np;
     GroupRecord &rec = tile[g / 2].g[g & 1];
     const GroupChans c = chans_of(a, g);
-    int dmin[kGroupMax], smax[kGroupMax], s0min = 0x7fffffff;
+    const float dms[2] = {dm[lane], dm[lane + 32]};
+    int s0[2], dmin[kGroupMax], smax[kGroupMax];
+    for (int h = 0; h < 2; ++h)
+        s0[h] = shift_of(dms[h], c.ds[0]);
     for (int i = 0; i < c.n; ++i) {
-        dmin[i] = 0x7fffffff;
-        smax[i] = 0;
+        const int sa = shift_of(dms[0], c.ds[i]), sb = shift_of(dms[1], c.ds[i]);
+        dmin[i] = __reduce_min_sync(kAll, min(sa - s0[0], sb - s0[1]));
+        smax[i] = __reduce_max_sync(kAll, max(sa, sb));
     }
-    for (int k = 0; k < kGroupDmCta; ++k) {
-        const int s0 = shift_of(dm[k], c.ds[0]);
-        s0min = min(s0min, s0);
-        for (int i = 0; i < c.n; ++i) {
-            const int s = shift_of(dm[k], c.ds[i]);
-            dmin[i] = min(dmin[i], s - s0);
-            smax[i] = max(smax[i], s);
-        }
-    }
-    const int ub = s0min & ~3;  // u = 0
+    const int ub = __reduce_min_sync(kAll, min(s0[0], s0[1])) & ~3;  // u = 0
     bool bad = false;
-    // The patterns: key, and the range of reference shifts.
-    uint32_t keys[kGroupTuples];
-    int lo[kGroupTuples], hi[kGroupTuples], nt = 0;
-    for (int k = 0; k < kGroupDmCta && !bad; ++k) {
-        const int u = shift_of(dm[k], c.ds[0]) - ub;
-        const uint32_t key = pattern_key(c, dm[k], u + ub, dmin, &bad);
-        int t = 0;
-        while (t < nt && keys[t] != key)
-            ++t;
-        if (t == kGroupTuples) {
+    uint32_t key[2];
+    for (int h = 0; h < 2; ++h)
+        key[h] = pattern_key(c, dms[h], s0[h], dmin, &bad);
+    // The patterns, ordered by key, so that neighbours fit a class; lane t has
+    // pattern t: key and range of reference shifts.
+    uint32_t tkey = 0;
+    int lo = 0, hi = 0, nt = 0;
+    bool open[2] = {true, true};
+    while (__any_sync(kAll, open[0] || open[1])) {
+        const uint32_t next =
+            __reduce_min_sync(kAll, min(open[0] ? key[0] : kAll, open[1] ? key[1] : kAll));
+        int l = 0x7fffffff, m = -1;
+        for (int h = 0; h < 2; ++h)
+            if (open[h] && key[h] == next) {
+                l = min(l, s0[h] - ub);
+                m = max(m, s0[h] - ub);
+                open[h] = false;
+            }
+        l = __reduce_min_sync(kAll, l);
+        m = __reduce_max_sync(kAll, m);
+        if (nt == kGroupTuples) {
             bad = true;
             break;
         }
-        if (t == nt) {
-            keys[nt] = key;
-            lo[nt] = hi[nt] = u;
-            ++nt;
+        if (lane == nt) {
+            tkey = next;
+            lo = l;
+            hi = m;
         }
-        lo[t] = min(lo[t], u);
-        hi[t] = max(hi[t], u);
-    }
-    // Ordered by key, so that neighbours fit a class.
-    for (int i = 1; i < nt; ++i) {
-        const uint32_t key = keys[i];
-        const int l = lo[i], h = hi[i];
-        int j = i - 1;
-        for (; j >= 0 && keys[j] > key; --j) {
-            keys[j + 1] = keys[j];
-            lo[j + 1] = lo[j];
-            hi[j + 1] = hi[j];
-        }
-        keys[j + 1] = key;
-        lo[j + 1] = l;
-        hi[j + 1] = h;
+        ++nt;
     }
     int phase[kGroupMax];  // byte of the staged row that u = 0 of offset 0 reads
     for (int i = 0; i < a.G; ++i) {
@@ -496,87 +493,115 @@ __global__ void __launch_bounds__(kPrepThreads) group_prep_kernel(const GroupPre
             if (start < 0 || r.bytes + 16 > a.rowcap)
                 bad = true;
         }
-        rec.rows[i] = r;
+        if (lane == 0)
+            rec.rows[i] = r;
     }
-    GroupHeader h = {};
-    int size = 0, top = 0;
-    uint32_t emin = 0, emax = 0;  // of the current class
-    for (int t = 0; t < nt && !bad; ++t) {
-        lo[t] &= ~3;
-        hi[t] = (hi[t] + kGroupTCta + 3) & ~3;
-        if (hi[t] > 0xffff)
-            bad = true;
-        GroupTuple &v = rec.tup[t];
-        v.lolen = (uint32_t)lo[t] | (uint32_t)(hi[t] - lo[t]) << 16;
-        v.at = size - 2 * lo[t];
-        // Does it fit the class so far?
+    const bool mine = lane < nt;
+    lo &= ~3;
+    hi = mine ? (hi + kGroupTCta + 3) & ~3 : lo;
+    if (hi > 0xffff)
+        bad = true;
+    const int len = hi - lo;
+    int size = 4 * len;  // of the arrays up to this lane's
+#pragma unroll
+    for (int o = 1; o < 32; o *= 2) {
+        const int v = __shfl_up_sync(kAll, size, o);
+        size += lane >= o ? v : 0;
+    }
+    const int before = size - 4 * len;
+    // Classes: each pattern joins the one before it if their offsets differ by
+    // at most 3 all told.  cls: this lane's class, base: its smallest offsets.
+    int ncls = 0, cls = -1;
+    uint32_t base = 0, emin = 0, emax = 0;
+    for (int t = 0; t < nt; ++t) {
+        const uint32_t k = __shfl_sync(kAll, tkey, t);
         bool fits = t > 0;
         uint32_t lo2 = 0, hi2 = 0;
         for (int i = 1; i < c.n; ++i) {
-            const uint32_t e = nibble(keys[t], i);
+            const uint32_t e = nibble(k, i);
             const uint32_t l = min(e, nibble(emin, i)), m = max(e, nibble(emax, i));
             fits = fits && m - l <= 3;
             lo2 |= l << (4 * i);
             hi2 |= m << (4 * i);
         }
-        if (fits) {
-            emin = lo2;
-            emax = hi2;
-        } else if (h.ncls == kGroupClasses) {
-            bad = true;
-            break;
-        } else {
-            ++h.ncls;
-            emin = emax = keys[t];
+        if (!fits) {
+            ++ncls;
+            lo2 = hi2 = k;
         }
-        const int k = h.ncls - 1;
-        h.cnt[k / 4] += 1u << (8 * (k % 4));
-        const int n = (int)((h.cnt[k / 4] >> (8 * (k % 4))) & 255u);
-        GroupClass cl = {};
-        for (int i = 0; i < c.n; ++i) {
-            const int p = phase[i] + (int)nibble(emin, i);
-            cl.at[i] = i * a.rowcap + (p & ~3);
-            cl.sh[i] = 0x3210u + 0x1111u * (uint32_t)(p & 3);
-        }
-        rec.cls[k] = cl;
-        for (int q = t - n + 1; q <= t; ++q) {  // the class's patterns so far
-            uint32_t e[4];
-            for (int i = 1; i < 4; ++i)
-                e[i] = nibble(keys[q], i) - nibble(emin, i);
-            rec.tup[q].a = 0x32103210u + 0x1111u * e[1] + 0x11110000u * e[2];
-            rec.tup[q].b = 0x3210u + 0x1111u * e[3] + (e[1] << 19) + (e[2] << 24) + (e[3] << 29);
-        }
-        size += 4 * (hi[t] - lo[t]);
-        top = max(top, hi[t]);
+        emin = lo2;
+        emax = hi2;
+        if (lane == t)
+            cls = ncls - 1;
+        if (cls == ncls - 1)
+            base = emin;
     }
-    h.nt = nt;
-    h.nunit = (top + kGroupUnit - 1) / kGroupUnit;
-    h.nch = c.n;
-    rec.head = h;
-    sizes[(int64_t)td * ng + g] = size;
-    // The DMs' words (from the group's first array; its place is added below).
-    for (int k = 0; k < kGroupDmCta && !bad; ++k) {
-        const int s0 = shift_of(dm[k], c.ds[0]);
-        const uint32_t key = pattern_key(c, dm[k], s0, dmin, &bad);
-        int at = 0;
-        for (int t = 0; t < nt && keys[t] != key; ++t)
-            at += 4 * (hi[t] - lo[t]);
-        for (int t = 0; t < nt; ++t)
-            if (keys[t] == key) {
-                const int u = s0 - ub - lo[t];
-                at += (u & 1) * 2 * (hi[t] - lo[t]) + (u >> 1) * 4;
+    if (ncls > kGroupClasses)
+        bad = true;
+    bad = __any_sync(kAll, bad);
+    if (bad) {
+        if (lane == 0) {
+            rec.head = GroupHeader{};
+            sizes[(int64_t)td * ng + g] = 0;
+            atomicExch(a.fail, 1);
+        }
+        return;
+    }
+    GroupHeader h = {};
+    for (int k = 0; k < ncls; ++k) {
+        const uint32_t in = __ballot_sync(kAll, cls == k);
+        h.cnt[k / 4] += (uint32_t)__popc(in) << (8 * (k % 4));
+        if (lane == __ffs(in) - 1) {
+            GroupClass cl = {};
+            for (int i = 0; i < c.n; ++i) {
+                const int p = phase[i] + (int)nibble(base, i);
+                cl.at[i] = i * a.rowcap + (p & ~3);
+                cl.sh[i] = 0x3210u + 0x1111u * (uint32_t)(p & 3);
             }
-        tile[g / 2].offs[k][g & 1] = at;
+            rec.cls[k] = cl;
+        }
     }
-    if (bad)
-        atomicExch(a.fail, 1);
+    if (mine) {
+        uint32_t e[4];
+        for (int i = 1; i < 4; ++i)
+            e[i] = nibble(tkey, i) - nibble(base, i);
+        GroupTuple &v = rec.tup[lane];
+        v.lolen = (uint32_t)lo | (uint32_t)len << 16;
+        v.at = before - 2 * lo;
+        v.a = 0x32103210u + 0x1111u * e[1] + 0x11110000u * e[2];
+        v.b = 0x3210u + 0x1111u * e[3] + (e[1] << 19) + (e[2] << 24) + (e[3] << 29);
+    }
+    const int top = __reduce_max_sync(kAll, mine ? hi : 0);
+    size = __shfl_sync(kAll, size, 31);
+    if (lane == 0) {
+        h.ncls = ncls;
+        h.nt = nt;
+        h.nunit = (top + kGroupUnit - 1) / kGroupUnit;
+        h.nch = c.n;
+        rec.head = h;
+        sizes[(int64_t)td * ng + g] = size;
+    }
+    // The DMs' words (from the group's first array; its place is added below).
+    int at[2] = {0, 0};
+    for (int t = 0; t < nt; ++t) {
+        const uint32_t k = __shfl_sync(kAll, tkey, t);
+        const int b = __shfl_sync(kAll, before, t), l = __shfl_sync(kAll, lo, t),
+                  n = __shfl_sync(kAll, len, t);
+        for (int q = 0; q < 2; ++q)
+            if (key[q] == k) {
+                const int u = s0[q] - ub - l;
+                at[q] = b + (u & 1) * 2 * n + (u >> 1) * 4;
+            }
+    }
+    for (int q = 0; q < 2; ++q)
+        tile[g / 2].offs[lane + 32 * q][g & 1] = at[q];
 }
 
 // The arrays' places: even pairs from the start of the array space, odd pairs
 // up to its end; two neighbours are held at once.
 __global__ void __launch_bounds__(kPrepThreads) group_place_kernel(const GroupPrep a,
                                                                    const int *sizes) {
-    const int td = blockIdx.y, g = blockIdx.x * kPrepThreads + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    const int td = blockIdx.y, g = (blockIdx.x * kPrepThreads + threadIdx.x) / 32;
     const int np = ((a.nchan + a.G - 1) / a.G + 1) / 2, ng = 2 * np;
     if (g >= ng)
         return;
@@ -587,10 +612,10 @@ __global__ void __launch_bounds__(kPrepThreads) group_place_kernel(const GroupPr
         atomicExch(a.fail, 1);
     const int off = ((g & 2) ? space - pair : 0) + ((g & 1) ? first : 0);
     GroupEntry &ent = a.entries[(int64_t)td * np + g / 2];
-    for (int k = 0; k < kGroupDmCta; ++k)
-        ent.offs[k][g & 1] += off;
-    for (int t = 0; t < ent.g[g & 1].head.nt; ++t)
-        ent.g[g & 1].tup[t].at += off;
+    ent.offs[lane][g & 1] += off;
+    ent.offs[lane + 32][g & 1] += off;
+    if (lane < ent.g[g & 1].head.nt)
+        ent.g[g & 1].tup[lane].at += off;
 }
 
 }  // namespace
@@ -614,7 +639,7 @@ GroupEntry *build_group_table(GroupPrep a, int dev) {
         int *sizes = reinterpret_cast<int *>(static_cast<uint8_t *>(mem) + table);
         a.fail = sizes + 2 * pairs;
         const unsigned ng = 2 * (unsigned)(pairs / (size_t)a.ntile_d);
-        const dim3 grid((ng + kPrepThreads - 1) / kPrepThreads, (unsigned)a.ntile_d);
+        const dim3 grid((ng + kPrepThreads / 32 - 1) / (kPrepThreads / 32), (unsigned)a.ntile_d);
         if (cudaMemsetAsync(a.fail, 0, sizeof(int), s) == cudaSuccess) {
             group_prep_kernel<<<grid, kPrepThreads, 0, s>>>(a, sizes);
             group_place_kernel<<<grid, kPrepThreads, 0, s>>>(a, sizes);
