@@ -164,7 +164,8 @@ extern "C" dd_status dd_execute_host(dd_plan_t p, const void *in_host, dd_dtype 
             const int64_t first = whole_rounds(p, dtype, edge);
             blocks.push_back(first);
             int64_t rest = nsamp_out - 2 * first;
-            for (int64_t m = (rest + mid - 1) / mid; m > 0; --m) {
+            while (rest > 0) {
+                const int64_t m = (rest + mid - 1) / mid;
                 blocks.push_back(m > 1 ? whole_rounds(p, dtype, rest / m) : rest);
                 rest -= blocks.back();
             }
