@@ -102,10 +102,10 @@ constexpr double kGain = 0.95;
 bool group_shape(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &dt,
                  int64_t nsamp_out, bool alone, GroupShape *out) {
     // The preferred tile shape stands for the library's choice; another shape
-    // set by the caller runs as such.
+    // set by the caller, or timed by the autotuner, runs as such.
     const dd_tiles pref = default_tiles(DD_U8);
     int dev = 0;
-    if (t != DD_U8 || (std::memcmp(&pref, &g.tiles, sizeof(pref)) != 0 && !tiles_open(p, t)) ||
+    if (t != DD_U8 || (std::memcmp(&pref, &g.tiles, sizeof(pref)) != 0 && !g.chosen) ||
         cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
         return false;
     const int sms = sm_count(dev);

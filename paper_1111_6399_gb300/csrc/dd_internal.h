@@ -98,6 +98,7 @@ struct Geometry {
     int smem = 0;         // dynamic shared memory per CTA
     int builders = 0;     // phase-builder warps (0 for FP32)
     int threads = 0;      // consumer warps + one producer warp + builder warps
+    bool chosen = false;  // by execution_geometry, not set or being measured
 };
 
 struct GroupShape;  // dd_group.h
@@ -172,9 +173,6 @@ dd_status execution_geometry(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, Geomet
 // Modelled time of an execution by the direct kernel, to compare lengths by
 // (microseconds, or rounds of tiles where the shape has been set).
 double execution_time(dd_plan_s *p, dd_dtype t, int64_t nsamp_out);
-
-// Neither the caller nor the autotuner has set the plan's shape.
-bool tiles_open(dd_plan_s *p, dd_dtype t);
 
 // Modelled time of the direct kernel in one of the shapes that
 // execution_geometry chooses from (-1 for another shape).

@@ -116,11 +116,6 @@ double direct_time_us(dd_dtype t, const dd_tiles &tl, int nchan, int ndm, int64_
     return -1.0;
 }
 
-bool tiles_open(dd_plan_s *p, dd_dtype t) {
-    std::lock_guard<std::mutex> lk(p->mu);
-    return p->tiles_open[t];
-}
-
 namespace {
 
 // The listed shape expected to finish first (-1: none fits), and its time.
@@ -159,6 +154,7 @@ dd_status execution_geometry(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, Geomet
                 it = p->geo.emplace(key, r).first;
             if (it != p->geo.end()) {
                 *g = it->second;
+                g->chosen = true;
                 return DD_OK;
             }
             // Its windows do not fit shared memory: passed over from now on.

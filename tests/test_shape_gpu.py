@@ -49,3 +49,37 @@ def test_chosen_shape_matches_oracle(built_lib, oracle_lib, kind, nchan, ndm, ns
                                     threads=True)
         bound = (66 + nchan / 60) * 2.0 ** -24 * mag
         assert np.all(np.abs(got[:, :ns].astype(np.float64) - want) <= bound)
+
+
+@pytest.mark.parametrize("kind,nchan,ndm,ns", [("u8", 96, 40, 57345), ("u8", 33, 301, 115000),
+                                               ("f32", 64, 20, 90001)])
+def test_host_blocks_equal_one_execution(built_lib, kind, nchan, ndm, ns):
+    """Several host blocks of whole tile rounds give what one launch gives
+    (integer values: exact in every type and shape)."""
+    rng = np.random.default_rng(ns)
+    plan = built_lib.Plan(nchan, 1400.0, -300.0 / nchan, 1e-4,
+                          rng.uniform(0.0, 60.0, size=ndm).astype(np.float32))
+    nin = ns + plan.maxshift
+    data = fb.random_filterbank(rng, nchan, nin, kind, pitch=(nin + 15) // 16 * 16)
+    x = torch.from_numpy(data).cuda()
+    out = torch.empty((ndm, (ns + 3) // 4 * 4), dtype=torch.float32, device="cuda")
+    plan.execute(x, out, nsamp_in=nin, nsamp_out=ns)
+    host = np.full((ndm, ns + 5), -7.0, dtype=np.float32)
+    plan.execute_host(data, host, nsamp_in=nin, nsamp_out=ns)
+    assert np.array_equal(host[:, :ns], out.cpu().numpy()[:, :ns])
+    assert np.all(host[:, ns:] == -7.0)
+
+
+def test_autotuner_times_the_shapes_themselves(built_lib):
+    """On a beam that the channel-group kernel takes, only the default shape
+    stands for it: 8-DM tiles, a sixth of its rate, are timed as such."""
+    dms = np.arange(260, dtype=np.float32) * 0.5
+    plan = built_lib.Plan(512, 1500.0, -30.0 / 512, 64e-6, dms)
+    ns = 61440
+    nin = (ns + plan.maxshift + 15) // 16 * 16
+    x = torch.zeros((512, nin), dtype=torch.uint8, device="cuda")
+    out = torch.empty((260, ns), dtype=torch.float32, device="cuda")
+    plan.execute(x, out, nsamp_in=nin, nsamp_out=ns)   # builds the table first
+    ms = {tuple(t): m for t, m in plan.autotune(x, out, nsamp_in=nin, nsamp_out=ns)}
+    assert ms[(1, 8, 1, 16, 4)] > 2.0 * ms[(4, 12, 1, 8, 8)] > 0.0
+    assert plan.get_tiles("u8") == min((m, t) for t, m in ms.items() if m >= 0)[1]
