@@ -113,7 +113,9 @@ int dd_plan_ndm(dd_plan_t plan);            /* -1 on NULL */
 /* Copy the FP32 dmshift table (nchan floats) to host memory. */
 dd_status dd_plan_dmshift(dd_plan_t plan, float *host_out);
 
-/* Tile shape the plan uses for dtype (default heuristic unless set).  */
+/* Tile shape of the plan for dtype (a default unless set or autotuned).  While
+ * it is the default, an execution may run in another shape that a count of
+ * tile rounds expects to finish earlier. */
 dd_status dd_plan_get_tiles(dd_plan_t plan, dd_dtype dtype, dd_tiles *tiles_out);
 
 /* Override the tile shape for dtype (validated: shared-memory fit, supported
@@ -150,13 +152,16 @@ dd_status dd_autotune(dd_plan_t plan, const void *in, dd_dtype dtype, int64_t in
  * Validation (DD_ERR_INVALID, nothing launched): alignment rules above,
  * in_pitch >= nsamp_in, out_pitch >= nsamp_out, nsamp_in large enough.
  * The first call on a device uploads the plan's tables (synchronous copy).
- * When the last DM tile of the plan's tile shape would be at most half full
+ * The tile shape is the plan's if it has been set (dd_plan_set_tiles,
+ * dd_autotune), else chosen by nchan, ndm, nsamp_out and dtype; results do not
+ * depend on it beyond FP32 rounding (uint8: not at all).
+ * When the last DM tile of that shape would be at most half full
  * and a count of tile rounds says it finishes earlier, the DMs of that tile
  * run as a second launch on a library-owned stream: it waits for an event
  * recorded on `stream` before the call's work, and `stream` waits for its
  * completion, so every later operation on `stream` sees the whole plane.
- * uint8 beams of the preferred tile shape (4 DMs x 8 words per thread, 12 DM
- * warps, 8-channel stages) whose neighbouring channels' shifts differ little
+ * uint8 beams whose shape has not been set (or is the default: 4 DMs x 8 words
+ * per thread, 12 DM warps, 8-channel stages) and whose neighbouring channels' shifts differ little
  * run in a kernel of its own tiles (64 DMs x 1024 samples) that sums groups of
  * channels once per shift pattern, where a count of tile rounds says it
  * finishes earlier; the sums are the same.  Its table (2.5 KB per 64 DMs and 8
@@ -238,8 +243,8 @@ dd_status dd_execute_detect(dd_plan_t plan, const void *in, dd_dtype dtype, int6
  * (channel c of spectrum t starts at bit (t*nchan + c)*nbits of the block;
  * bit b is bit b%8 of byte b/8).
  *   in:  device pointer to nsamp*nchan*nbits/8 bytes; any alignment.  Input
- *        that is 16-byte aligned, with nchan a multiple of 128 and spectra a
- *        multiple of 16 bytes, takes the faster tiled path.
+ *        on 16, 8 or 4 bytes whose spectra are a multiple of as many takes the
+ *        faster tiled path.
  *   out: device uint8 [nchan][out_pitch], 16-byte aligned, out_pitch >= nsamp
  *        and a multiple of 16; out[c][t] = the sample (0 .. 2^nbits - 1, not
  *        rescaled).  Columns t >= nsamp are left untouched.
