@@ -110,12 +110,14 @@ bool group_shape(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &d
         return false;
     const int sms = sm_count(dev);
     const int64_t tiles = (nsamp_out + g.t_cta - 1) / g.t_cta * g.ntile_d;
-    if (sms <= 0 || (alone && tiles <= sms))
-        return false;  // one round of the direct kernel's tiles
+    if (sms <= 0)
+        return false;
     // Time of the direct kernel: in rounds of tiles over the SMs, or, as one of
     // many beams, its share of them.
     double direct = direct_time_us(t, g.tiles, p->nchan, p->ndm, nsamp_out, sms);
-    if (direct < 0)
+    // A table costs a plan's first execution about 110 us (35 of them for the
+    // samples below), more than shorter beams gain in many.
+    if (direct < (alone ? 100.0 : 0.0))
         return false;
     if (!alone)
         direct *= (double)tiles / sms / (double)((tiles + sms - 1) / sms);

@@ -100,10 +100,30 @@ double shape_time_us(dd_dtype t, const ShapeCost &c, int nchan, int ndm, int64_t
                      int sms) {
     const int64_t d = c.tiles.dm_per_thread * c.tiles.dm_warps;
     const int64_t len = (int64_t)warp_span(t, c.tiles.words_per_thread) * c.tiles.time_warps;
-    const int64_t n = (ndm + d - 1) / d * ((nsamp_out + len - 1) / len);
+    const int64_t nt = (nsamp_out + len - 1) / len, n = (ndm + d - 1) / d * nt;
     const int64_t slots = (int64_t)sms * c.resident;
-    return (double)((n + slots - 1) / slots) *
-           std::max(0.5 * c.us64, c.us64 + (c.us512 - c.us64) * (nchan - 64) / 448.0);
+    // The last of many rounds, partly filled, overlaps the others (their tiles
+    // are out of step): 1428 and 1344 tiles of 64 channels took 9.4 and 9.1
+    // rounds on 152 SMs, 476 tiles of 1422 channels still 4.
+    auto rounds_of = [&](int64_t tiles) {
+        const double whole = (double)((tiles + slots - 1) / slots),
+                     part = (double)tiles / (double)slots;
+        return part + (whole - part) * std::min(1.0, 4.0 / whole);
+    };
+    double rounds = rounds_of(n);
+    // Few DMs left by the preferred FP16 / FP32 shape may run as a launch of
+    // their own beside the last round (tail_geometry): 512 channels x 100 DMs
+    // x 65536 FP32 take 500 us as 96 + 4 DMs, 522 in 32-DM tiles.  (uint8 beams
+    // of that kind go to the channel groups as often as not.)
+    const int64_t rem = ndm % d;
+    if (t != DD_U8 && &c == &shape_costs(t)[0] && ndm >= d && rem > 0 && 2 * rem <= d) {
+        const int64_t full = ndm / d * nt, free = (full + slots - 1) / slots * slots - full,
+                      dmw = (rem + c.tiles.dm_per_thread - 1) / c.tiles.dm_per_thread,
+                      tl = len * std::max<int64_t>(1, c.tiles.dm_warps / dmw);
+        if ((nsamp_out + tl - 1) / tl <= free)
+            rounds = std::min(rounds, rounds_of(full) + (double)rem / (double)d);
+    }
+    return rounds * std::max(0.5 * c.us64, c.us64 + (c.us512 - c.us64) * (nchan - 64) / 448.0);
 }
 
 }  // namespace
@@ -125,7 +145,9 @@ int fastest_shape(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, int sms, double *
     for (int i = 0; i < (int)shapes.size(); ++i) {
         if (p->shape_unfit[t] >> i & 1u)
             continue;
-        const double u = shape_time_us(t, shapes[i], p->nchan, p->ndm, nsamp_out, sms);
+        // (2 % in favour of the preferred shape, the first.)
+        const double u = shape_time_us(t, shapes[i], p->nchan, p->ndm, nsamp_out, sms) *
+                         (i > 0 ? 1.02 : 1.0);
         if (best < 0 || u < *us) {
             best = i;
             *us = u;
