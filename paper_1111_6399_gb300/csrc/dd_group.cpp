@@ -113,14 +113,14 @@ bool group_shape(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &d
     if (sms <= 0)
         return false;
     // Time of the direct kernel: in rounds of tiles over the SMs, or, as one of
-    // many beams, its share of them.
-    double direct = direct_time_us(t, g.tiles, p->nchan, p->ndm, nsamp_out, sms);
+    // many beams, its share of them (of the time of one tile's round).
+    const double direct =
+        alone ? direct_time_us(t, g.tiles, p->nchan, p->ndm, nsamp_out, sms)
+              : direct_time_us(t, g.tiles, p->nchan, 1, 1, sms) * (double)tiles / sms;
     // A table costs a plan's first execution about 110 us (35 of them for the
     // samples below), more than shorter beams gain in many.
     if (direct < (alone ? 100.0 : 0.0))
         return false;
-    if (!alone)
-        direct *= (double)tiles / sms / (double)((tiles + sms - 1) / sms);
     std::lock_guard<std::mutex> lk(p->mu);
     auto it = p->group.find(dev);
     if (it == p->group.end()) {
@@ -132,8 +132,10 @@ bool group_shape(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &d
         double spread = 0;
         const double most = *std::max_element(p->dmshift.begin(), p->dmshift.end());
         for (int a = 0; a < p->ndm; a += kGroupDmCta)
-            spread = std::max(spread, most * ((double)p->dm_sorted[(size_t)std::min(a + kGroupDmCta, p->ndm) - 1] -
-                                              (double)p->dm_sorted[(size_t)a]));
+            spread = std::max(
+                spread,
+                most * ((double)p->dm_sorted[(size_t)std::min(a + kGroupDmCta, p->ndm) - 1] -
+                        (double)p->dm_sorted[(size_t)a]));
         if (spread < 8192) {
             r->rowcap = (kGroupTCta + (int)spread + 64 + 15) / 16 * 16;
             for (int G : {4, 3}) {
