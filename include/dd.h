@@ -154,7 +154,8 @@ dd_status dd_autotune(dd_plan_t plan, const void *in, dd_dtype dtype, int64_t in
  * The first call on a device uploads the plan's tables (synchronous copy).
  * The tile shape is the plan's if it has been set (dd_plan_set_tiles,
  * dd_autotune), else chosen by nchan, ndm, nsamp_out and dtype; results do not
- * depend on it beyond FP32 rounding (uint8: not at all).
+ * depend on it, bit for bit (FP16/FP32: among shapes whose chan_per_stage
+ * divides 48, as in every shape that the library chooses or tunes among).
  * When the last DM tile of that shape would be at most half full
  * and a count of tile rounds says it finishes earlier, the DMs of that tile
  * run as a second launch on a library-owned stream: it waits for an event

@@ -359,7 +359,7 @@ static std::vector<dd_tiles> tune_candidates(dd_dtype t) {
                     if (w > dd::max_consumer_warps(dthr, nw) || w < 8)
                         continue;
                     for (int cs : css) {
-                        const int limit = t == DD_U8 ? dd::kSwarChannels : dd::kFloatBlock;
+                        const int limit = t == DD_U8 ? dd::kSwarChannels : dd::kFloatStage;
                         if (cs > limit)
                             continue;
                         out.push_back(dd_tiles{dthr, dw, wt, cs, nw});

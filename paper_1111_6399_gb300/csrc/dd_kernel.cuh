@@ -32,7 +32,7 @@
 //    widened into the FP32 output (exact: every sum < 2^24).  Per word and two
 //    channels: 2 LDS + 1 IADD3 (ALU) + 2 PRMT (ALU) + 2 IMAD (FMA pipe), which
 //    balances the integer ALU and FMA pipes.
-//  * FP16/FP32 sums: FP32 partials over blocks of 64 channels, combined into a
+//  * FP16/FP32 sums: FP32 partials over blocks of 48 channels, combined into a
 //    running sum with TwoSum compensation (error ~1e-7 of sum |in|).
 //
 // Work distribution.  The producer decides which tile the CTA works on and

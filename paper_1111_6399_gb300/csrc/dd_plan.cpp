@@ -249,7 +249,7 @@ dd_status make_geometry_range(dd_plan_s *p, dd_dtype t, const dd_tiles &tl, int 
                                         " for this dm_per_thread and words_per_thread");
     if (tl.chan_per_stage < 4 || tl.chan_per_stage > 64 || (tl.chan_per_stage & 3))
         return fail(DD_ERR_INVALID, "tile shape: chan_per_stage must be a multiple of 4, 4..64");
-    const int limit = (t == DD_U8) ? kSwarChannels : kFloatBlock;
+    const int limit = (t == DD_U8) ? kSwarChannels : kFloatStage;
     if (tl.chan_per_stage > limit)
         return fail(DD_ERR_INVALID, "tile shape: chan_per_stage must not exceed the "
                                     "accumulation block (256 for uint8, 64 otherwise)");
