@@ -11,11 +11,6 @@
 namespace dd {
 namespace {
 
-int shift_host(float dm, float ds) {
-    volatile float prod = dm * ds;  // one FP32 multiply, round to nearest even
-    return (int)prod;
-}
-
 // Patterns of sampled (DM tile, group) pairs: 3 tiles x 12 groups spread over
 // the plan.
 struct Sample {
@@ -42,10 +37,10 @@ Sample sample_patterns(const dd_plan_s *p, int G) {
             int lo[kGroupTuples], hi[kGroupTuples], nt = 0, s_lo = 0x7fffffff, s_hi = 0;
             for (int k = 0; k < kGroupDmCta; ++k) {
                 const float dm = p->dm_sorted[(size_t)std::min(td * kGroupDmCta + k, p->ndm - 1)];
-                const int s0 = shift_host(dm, ds[ref]);
+                const int s0 = trunc_product(dm, ds[ref]);
                 int64_t key = 0;
                 for (int i = 0; i < n; ++i)
-                    key = key << 15 | ((shift_host(dm, ds[i]) - s0) & 0x7fff);
+                    key = key << 15 | ((trunc_product(dm, ds[i]) - s0) & 0x7fff);
                 int t = nt;
                 while (t > 0 && keys[t - 1] != key)
                     --t;
@@ -86,10 +81,6 @@ double group_clocks(const Sample &s, int G) {
     return users + 3.9 * (3 * units + 4.5 * arrays / G + units);
 }
 
-// The direct kernel's times are measured where a 64-DM tile spans up to 430
-// samples (590 clocks per channel and tile of its preferred shape); wider
-// windows cost it more (729 clocks at 860 samples).
-double spread_factor(double spread) { return 1.0 + 0.32 / 590 * std::max(0.0, spread - 430.0); }
 // Prologue and epilogue of a tile, clocks.
 constexpr double kTileClocks = 10000;
 constexpr double kClocksPerUs = 2070;
@@ -114,9 +105,8 @@ bool group_shape(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &d
         return false;
     // Time of the direct kernel: in rounds of tiles over the SMs, or, as one of
     // many beams, its share of them (of the time of one tile's round).
-    const double direct =
-        alone ? direct_time_us(t, g.tiles, p->nchan, p->ndm, nsamp_out, sms)
-              : direct_time_us(t, g.tiles, p->nchan, 1, 1, sms) * (double)tiles / sms;
+    const double direct = alone ? direct_time_us(p, t, g.tiles, nsamp_out, sms)
+                                : direct_tile_us(p, t, g.tiles) * (double)tiles / sms;
     // A table costs a plan's first execution about 110 us (35 of them for the
     // samples below), more than shorter beams gain in many.
     if (direct < (alone ? 100.0 : 0.0))
@@ -144,7 +134,6 @@ bool group_shape(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &d
                 if (s.fits && kGroupRaw * group_raw_bytes(G, r->rowcap) < kGroupSmem / 2 &&
                     16.0 * s.nt * (kGroupTCta + s.reach) < group_array_bytes(G, r->rowcap)) {
                     r->sizes.push_back({G, group_clocks(s, G)});
-                    r->spread = s.spread;
                 }
             }
             std::sort(r->sizes.begin(), r->sizes.end(),
@@ -156,7 +145,7 @@ bool group_shape(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &d
     const double n = (double)group_tiles(r, nsamp_out) / sms;
     while (!r.sizes.empty() &&
            (alone ? std::ceil(n) : n) * (p->nchan * r.sizes[0].clk + kTileClocks) / kClocksPerUs <=
-               kGain * spread_factor(r.spread) * direct) {
+               kGain * direct) {
         if (!r.entries) {
             GroupPrep a;
             a.dmshift = dt.dmshift;

@@ -118,7 +118,6 @@ struct GroupArgs {
 // Grouped execution of a plan on one device.
 struct GroupShape {
     int ntile_d = 0, rowcap = 0;
-    double spread = 0;              // reference shifts a tile spans, on average (samples)
     // Group sizes that may serve, best first: channels, modelled SM clocks per
     // channel and tile.  Once a table is built, its size is the only one.
     struct Size {

@@ -4,6 +4,7 @@
 
 #include <cuda_runtime_api.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <map>
 #include <memory>
@@ -31,6 +32,14 @@ struct Range {
 inline int elem_size(dd_dtype t) { return t == DD_U8 ? 1 : (t == DD_F16 ? 2 : 4); }
 inline int warp_span(dd_dtype t, int words) { return 32 * words * (4 / elem_size(t)); }
 inline int phases(dd_dtype t) { return 4 / elem_size(t); }
+inline bool valid_dtype(dd_dtype t) { return t == DD_U8 || t == DD_F16 || t == DD_F32; }
+
+// The shift of a channel: one FP32 multiply, rounded to nearest even, then
+// truncated.
+inline int trunc_product(float dm, float ds) {
+    volatile float prod = dm * ds;
+    return (int)prod;
+}
 
 // Channels summed into 16-bit SWAR lanes before they are widened (uint8):
 // 256 * 255 = 65280 fits a 16-bit lane.
@@ -112,6 +121,11 @@ struct Geometry {
 
 struct GroupShape;  // dd_group.h
 
+struct ShapeFit {
+    int stages = 0;    // of the ring (0: the windows do not fit)
+    int resident = 1;  // CTAs on an SM
+};
+
 }  // namespace dd
 
 struct dd_plan_s {
@@ -128,7 +142,8 @@ struct dd_plan_s {
     std::map<int, dd::DevTables> dev;      // per CUDA device
     bool tiles_open[3] = {true, true, true};  // executions may choose, until set
     std::map<uint64_t, dd::Geometry> geo;  // per (dtype, tiles) key
-    uint32_t shape_unfit[3] = {0, 0, 0};   // shapes found not to fit, a bit each
+    std::vector<dd::ShapeFit> shape_fit[3];  // of the listed shapes (dd_shape.cpp), on first use
+    uint32_t shape_unfit[3] = {0, 0, 0};     // shapes found not to fit, a bit each
     // Remainder-DM launch per (dtype, tiles) key: (found, geometry).
     std::map<uint64_t, std::pair<bool, dd::Geometry>> tail_geo;
     std::map<int, std::shared_ptr<dd::GroupShape>> group;  // grouped execution, per device
@@ -145,6 +160,22 @@ dd_status fail(dd_status st, const std::string &msg);
 // stage, in the order the kernel lays them out, and 16 bytes for the
 // epilogue of fused detection.
 int64_t ring_smem(const Geometry &g, int64_t stage_bytes, int n);
+
+// Geometry of a tile shape before its windows are known, and its ring (four
+// stages, or as many as fit) for windows of `widest` bytes: false if not even
+// two stages of *smem bytes in all fit.
+Geometry tile_geometry(dd_dtype t, const dd_tiles &tl);
+bool ring_layout(Geometry *r, int64_t widest, int64_t *smem);
+
+// CTAs of `smem` bytes of dynamic shared memory that an SM holds (228 KB, 1 KB
+// per CTA reserved by the system).
+inline int resident_ctas(int smem) { return std::max(1, 233472 / (smem + 1024)); }
+
+inline uint64_t geo_key(dd_dtype t, const dd_tiles &tl) {
+    return ((uint64_t)t << 60) | ((uint64_t)tl.words_per_thread << 48) |
+           ((uint64_t)tl.dm_per_thread << 36) | ((uint64_t)tl.dm_warps << 24) |
+           ((uint64_t)tl.time_warps << 12) | (uint64_t)tl.chan_per_stage;
+}
 
 // Host checks of a beam's layout shared by the entry points that run one
 // beam: dtype, sample counts (nsamp_in >= nsamp_out + maxshift), pitches at
@@ -184,9 +215,10 @@ dd_status execution_geometry(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, Geomet
 double execution_time(dd_plan_s *p, dd_dtype t, int64_t nsamp_out);
 
 // Modelled time of the direct kernel in one of the shapes that
-// execution_geometry chooses from (-1 for another shape).
-double direct_time_us(dd_dtype t, const dd_tiles &tl, int nchan, int ndm, int64_t nsamp_out,
-                      int sms);
+// execution_geometry chooses from (-1 for another shape), and of one of its
+// tiles, alone on an SM.
+double direct_time_us(dd_plan_s *p, dd_dtype t, const dd_tiles &tl, int64_t nsamp_out, int sms);
+double direct_tile_us(dd_plan_s *p, dd_dtype t, const dd_tiles &tl);
 
 // Launch shape for the DMs of the last, partly filled DM tile of geometry g,
 // run as a launch of their own (see dd_plan.cpp); cached per tile shape.

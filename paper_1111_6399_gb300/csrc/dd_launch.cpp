@@ -34,11 +34,6 @@ SideStream g_side[64];
 // windows are staged for fewer DMs and its stages hold fewer channels
 // (measured 1.33 on the L-band beam: 0.415 ms against 0.312 ms).
 constexpr double kTailCost = 1.4;
-// Shared memory of an SM available to resident CTAs (228 KB less 1 KB per
-// CTA the system reserves).
-constexpr int kSmemPerSm = 233472;
-
-int resident(const Geometry &g) { return std::max(1, kSmemPerSm / (g.smem + 1024)); }
 
 // Whether running the remainder DMs as their own launch finishes earlier than
 // padding the last DM tile, in units of one main tile's time, with CTAs
@@ -49,7 +44,7 @@ int resident(const Geometry &g) { return std::max(1, kSmemPerSm / (g.smem + 1024
 // start of its last round on.
 bool split_pays(const Geometry &g, const Geometry &gt, int64_t ntile_t, int64_t ntile_t_tail,
                 int sms) {
-    const int64_t slots = (int64_t)sms * resident(g);
+    const int64_t slots = (int64_t)sms * resident_ctas(g.smem);
     if (slots <= 0)
         return false;
     const int64_t n_pad = ntile_t * g.ntile_d;

@@ -27,19 +27,6 @@ std::atomic<int64_t> g_launches{0};
 
 constexpr double kDispersionConst = 4148.808;  // s MHz^2 / (pc cm^-3)
 
-int trunc_product(float dm, float ds) {
-    volatile float prod = dm * ds;  // one FP32 multiply, round to nearest even
-    return (int)prod;
-}
-
-uint64_t geo_key(dd_dtype t, const dd_tiles &tl) {
-    return ((uint64_t)t << 60) | ((uint64_t)tl.words_per_thread << 48) |
-           ((uint64_t)tl.dm_per_thread << 36) | ((uint64_t)tl.dm_warps << 24) |
-           ((uint64_t)tl.time_warps << 12) | (uint64_t)tl.chan_per_stage;
-}
-
-bool valid_dtype(dd_dtype t) { return t == DD_U8 || t == DD_F16 || t == DD_F32; }
-
 }  // namespace
 
 namespace dd {
@@ -57,149 +44,6 @@ dd_tiles default_tiles(dd_dtype t) {
     case DD_F16: return dd_tiles{4, 12, 1, 12, 8};
     default:     return dd_tiles{4, 12, 1, 16, 8};
     }
-}
-
-namespace {
-
-// Tile shapes an execution chooses from, with the time of one round of tiles
-// (one CTA per SM, or `resident`) at 64 and 512 channels in microseconds:
-// each shape run for 8 rounds on a 300 MHz band at 1.5 GHz with unit DM
-// steps.  Large beams take the shape of the least time per output (the
-// preferred one, or one DM column more where that saves a round); small ones
-// a shape whose tiles are all resident at once.  With the preferred shape
-// alone, 64 channels x 64 DMs x 8192 samples took 29 us (16 CTAs on 152 SMs)
-// against 15, and 512 x 200 x 8192 took 153 against 71.
-struct ShapeCost {
-    dd_tiles tiles;
-    int resident;
-    double us64, us512;
-};
-const std::vector<ShapeCost> &shape_costs(dd_dtype t) {
-    static const std::vector<ShapeCost> u8 = {
-        {{4, 12, 1, 8, 8}, 1, 25.2, 155.0},  {{4, 13, 1, 8, 8}, 1, 26.8, 163.7},
-        {{4, 8, 1, 8, 8}, 1, 21.1, 118.8},   {{2, 16, 1, 8, 8}, 1, 19.3, 110.0},
-        {{2, 13, 1, 8, 8}, 1, 17.3, 98.0},   {{2, 8, 1, 12, 8}, 1, 15.0, 76.4},
-        {{4, 8, 1, 16, 4}, 1, 14.8, 72.8},   {{2, 16, 1, 16, 4}, 1, 14.3, 75.1},
-        {{2, 13, 1, 16, 4}, 1, 12.8, 66.3},  {{2, 8, 1, 16, 4}, 1, 11.8, 60.4},
-        {{1, 8, 1, 16, 4}, 1, 10.8, 58.0}};
-    static const std::vector<ShapeCost> f16 = {
-        {{4, 12, 1, 12, 8}, 1, 24.0, 133.0}, {{4, 8, 1, 12, 8}, 1, 19.3, 100.6},
-        {{2, 8, 1, 16, 8}, 1, 13.9, 75.6},   {{4, 8, 1, 16, 4}, 1, 13.8, 72.4},
-        {{2, 16, 1, 16, 4}, 1, 13.8, 80.9},  {{2, 8, 1, 16, 4}, 1, 11.2, 64.6},
-        {{1, 8, 1, 16, 4}, 2, 11.5, 69.0}};
-    static const std::vector<ShapeCost> f32 = {
-        {{4, 12, 1, 16, 8}, 1, 18.6, 113.4}, {{4, 6, 2, 16, 8}, 1, 18.4, 112.7},
-        {{4, 13, 1, 12, 8}, 1, 23.0, 128.8}, {{4, 10, 1, 16, 8}, 1, 16.2, 95.5},
-        {{4, 8, 1, 16, 8}, 1, 14.5, 81.6},   {{2, 16, 1, 16, 8}, 1, 14.0, 85.8},
-        {{2, 8, 1, 16, 8}, 1, 10.5, 61.5},   {{2, 8, 1, 24, 4}, 1, 9.2, 52.0},
-        {{1, 8, 1, 24, 4}, 2, 9.8, 54.0}};
-    return t == DD_U8 ? u8 : t == DD_F16 ? f16 : f32;
-}
-
-double shape_time_us(dd_dtype t, const ShapeCost &c, int nchan, int ndm, int64_t nsamp_out,
-                     int sms) {
-    const int64_t d = c.tiles.dm_per_thread * c.tiles.dm_warps;
-    const int64_t len = (int64_t)warp_span(t, c.tiles.words_per_thread) * c.tiles.time_warps;
-    const int64_t nt = (nsamp_out + len - 1) / len, n = (ndm + d - 1) / d * nt;
-    const int64_t slots = (int64_t)sms * c.resident;
-    // The last of many rounds, partly filled, overlaps the others (their tiles
-    // are out of step): 1428 and 1344 tiles of 64 channels took 9.4 and 9.1
-    // rounds on 152 SMs, 476 tiles of 1422 channels still 4.
-    auto rounds_of = [&](int64_t tiles) {
-        const double whole = (double)((tiles + slots - 1) / slots),
-                     part = (double)tiles / (double)slots;
-        return part + (whole - part) * std::min(1.0, 4.0 / whole);
-    };
-    double rounds = rounds_of(n);
-    // Few DMs left by the preferred FP16 / FP32 shape may run as a launch of
-    // their own beside the last round (tail_geometry): 512 channels x 100 DMs
-    // x 65536 FP32 take 500 us as 96 + 4 DMs, 522 in 32-DM tiles.  (uint8 beams
-    // of that kind go to the channel groups as often as not.)
-    const int64_t rem = ndm % d;
-    if (t != DD_U8 && &c == &shape_costs(t)[0] && ndm >= d && rem > 0 && 2 * rem <= d) {
-        const int64_t full = ndm / d * nt, free = (full + slots - 1) / slots * slots - full,
-                      dmw = (rem + c.tiles.dm_per_thread - 1) / c.tiles.dm_per_thread,
-                      tl = len * std::max<int64_t>(1, c.tiles.dm_warps / dmw);
-        if ((nsamp_out + tl - 1) / tl <= free)
-            rounds = std::min(rounds, rounds_of(full) + (double)rem / (double)d);
-    }
-    return rounds * std::max(0.5 * c.us64, c.us64 + (c.us512 - c.us64) * (nchan - 64) / 448.0);
-}
-
-}  // namespace
-
-double direct_time_us(dd_dtype t, const dd_tiles &tl, int nchan, int ndm, int64_t nsamp_out,
-                      int sms) {
-    for (const ShapeCost &c : shape_costs(t))
-        if (std::memcmp(&c.tiles, &tl, sizeof(tl)) == 0)
-            return shape_time_us(t, c, nchan, ndm, nsamp_out, sms);
-    return -1.0;
-}
-
-namespace {
-
-// The listed shape expected to finish first (-1: none fits), and its time.
-int fastest_shape(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, int sms, double *us) {
-    const std::vector<ShapeCost> &shapes = shape_costs(t);
-    int best = -1;
-    for (int i = 0; i < (int)shapes.size(); ++i) {
-        if (p->shape_unfit[t] >> i & 1u)
-            continue;
-        // (2 % in favour of the preferred shape, the first.)
-        const double u = shape_time_us(t, shapes[i], p->nchan, p->ndm, nsamp_out, sms) *
-                         (i > 0 ? 1.02 : 1.0);
-        if (best < 0 || u < *us) {
-            best = i;
-            *us = u;
-        }
-    }
-    return best;
-}
-
-}  // namespace
-
-dd_status execution_geometry(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, Geometry *g) {
-    int dev = 0;
-    int sms = 0;
-    if (valid_dtype(t) && cudaGetDevice(&dev) == cudaSuccess && (sms = sm_count(dev)) > 0) {
-        std::lock_guard<std::mutex> lk(p->mu);
-        while (p->tiles_open[t]) {
-            double us = 0;
-            const int best = fastest_shape(p, t, nsamp_out, sms, &us);
-            if (best < 0)
-                break;
-            const dd_tiles &tiles = shape_costs(t)[(size_t)best].tiles;
-            const uint64_t key = geo_key(t, tiles);
-            auto it = p->geo.find(key);
-            Geometry r;
-            if (it == p->geo.end() && make_geometry(p, t, tiles, &r) == DD_OK)
-                it = p->geo.emplace(key, r).first;
-            if (it != p->geo.end()) {
-                *g = it->second;
-                g->chosen = true;
-                return DD_OK;
-            }
-            // Its windows do not fit shared memory: passed over from now on.
-            p->shape_unfit[t] |= 1u << best;
-        }
-    }
-    return plan_geometry(p, t, g);
-}
-
-double execution_time(dd_plan_s *p, dd_dtype t, int64_t nsamp_out) {
-    int dev = 0;
-    const int sms = cudaGetDevice(&dev) == cudaSuccess ? std::max(1, sm_count(dev)) : 1;
-    {
-        std::lock_guard<std::mutex> lk(p->mu);
-        double us = 0;
-        if (p->tiles_open[t] && fastest_shape(p, t, nsamp_out, sms, &us) >= 0)
-            return us;
-    }
-    Geometry g;
-    if (plan_geometry(p, t, &g) != DD_OK)
-        return 1.0;
-    const int64_t n = (int64_t)g.ntile_d * ((nsamp_out + g.t_cta - 1) / g.t_cta);
-    return (double)((n + sms - 1) / sms);
 }
 
 std::vector<dd_tiles> auto_tiles(dd_dtype t) {
@@ -224,6 +68,39 @@ int64_t ring_smem(const Geometry &g, int64_t stage_bytes, int n) {
     // + 16: the epilogue barrier and flags of fused detection
     return n * stage_bytes + table + n * (kStageMeta + rowinfo) + g.zero_bytes + 24 * (int64_t)n +
            16;
+}
+
+Geometry tile_geometry(dd_dtype t, const dd_tiles &tl) {
+    Geometry r;
+    r.tiles = tl;
+    r.elem = elem_size(t);
+    r.nph = phases(t);
+    r.span = warp_span(t, tl.words_per_thread);
+    r.dm_cta = tl.dm_per_thread * tl.dm_warps;
+    r.t_cta = r.span * tl.time_warps;
+    return r;
+}
+
+bool ring_layout(Geometry *r, int64_t widest, int64_t *smem) {
+    const int64_t wp = widest + 16;
+    const int64_t zero_bytes = ((int64_t)r->elem * r->t_cta + 16 + 15) / 16 * 16;
+    // Per stage: the staged rows (every byte phase), the producer's offset
+    // table (one int per staged row and DM of the CTA), a stage record and,
+    // with phases to build, the bytes staged per row; then the zero row and
+    // three mbarriers per stage.
+    const int64_t stage_bytes = (int64_t)r->tiles.chan_per_stage * r->nph * wp;
+    r->zero_bytes = (int)zero_bytes;
+    int nst = 4;
+    while (nst > 2 && ring_smem(*r, stage_bytes, nst) > kMaxSmem)
+        --nst;
+    *smem = ring_smem(*r, stage_bytes, nst);
+    if (*smem > kMaxSmem)
+        return false;
+    r->wp = (int)wp;
+    r->stage_bytes = (int)stage_bytes;
+    r->nstages = nst;
+    r->smem = (int)*smem;
+    return true;
 }
 
 dd_status make_geometry(dd_plan_s *p, dd_dtype t, const dd_tiles &tl, Geometry *g) {
@@ -258,13 +135,7 @@ dd_status make_geometry_range(dd_plan_s *p, dd_dtype t, const dd_tiles &tl, int 
     // DMs per CTA.
     if (dthr * tl.dm_warps > kMaxDmPerCta)
         return fail(DD_ERR_INVALID, "tile shape: dm_per_thread*dm_warps must be <= 64");
-    Geometry r;
-    r.tiles = tl;
-    r.elem = elem_size(t);
-    r.nph = phases(t);
-    r.span = warp_span(t, nw);
-    r.dm_cta = dthr * tl.dm_warps;
-    r.t_cta = r.span * tl.time_warps;
+    Geometry r = tile_geometry(t, tl);
     r.threads = 32 * tl.dm_warps * tl.time_warps;
     r.ntile_d = (nd + r.dm_cta - 1) / r.dm_cta;
     // Widest staged window (bytes) over every DM tile and channel: the CTA at
@@ -284,28 +155,11 @@ dd_status make_geometry_range(dd_plan_s *p, dd_dtype t, const dd_tiles &tl, int 
             widest = std::max(widest, w);
         }
     }
-    const int64_t wp = widest + 16;
-    const int64_t zero_bytes = ((int64_t)r.elem * r.t_cta + 16 + 15) / 16 * 16;
-    // Per stage: the staged rows (every byte phase), the producer's offset
-    // table (one int per staged row and DM of the CTA), a stage record and,
-    // with phases to build, the bytes staged per row; then the zero row and
-    // three mbarriers per stage.
-    const int64_t stage_bytes = (int64_t)tl.chan_per_stage * r.nph * wp;
-    r.zero_bytes = (int)zero_bytes;
-    auto smem_for = [&](int64_t n) { return ring_smem(r, stage_bytes, (int)n); };
-    int nst = 4;
-    while (nst > 2 && smem_for(nst) > kMaxSmem)
-        --nst;
-    const int64_t smem = smem_for(nst);
-    if (smem > kMaxSmem)
+    int64_t smem = 0;
+    if (!ring_layout(&r, widest, &smem))
         return fail(DD_ERR_INVALID, "tile shape: staged window needs " + std::to_string(smem) +
                                         " bytes of shared memory (limit 232448); use fewer "
                                         "channels per stage or fewer DMs per CTA");
-    r.wp = (int)wp;
-    r.stage_bytes = (int)stage_bytes;
-    r.nstages = nst;
-    r.zero_bytes = (int)zero_bytes;
-    r.smem = (int)smem;
     // Two builder warps: with one, building a stage (about 3 shared-memory
     // ops per staged byte, queued behind the consumers' loads) can take
     // longer than consuming it.
@@ -495,7 +349,7 @@ dd_status dd_plan(int nchan, double fch1_mhz, double foff_mhz, double tsamp_s,
     // if the table were not monotone.
     int64_t s = 0;
     for (int c = 0; c < nchan; ++c)
-        s = std::max<int64_t>(s, trunc_product(p->dm_sorted.back(), p->dmshift[c]));
+        s = std::max<int64_t>(s, dd::trunc_product(p->dm_sorted.back(), p->dmshift[c]));
     p->maxshift = s;
     for (int t = 0; t < 3; ++t)
         p->tiles[t] = dd::default_tiles((dd_dtype)t);
@@ -534,7 +388,7 @@ dd_status dd_plan_dmshift(dd_plan_t p, float *host_out) {
 }
 
 dd_status dd_plan_get_tiles(dd_plan_t p, dd_dtype t, dd_tiles *out) {
-    if (!p || !out || !valid_dtype(t))
+    if (!p || !out || !dd::valid_dtype(t))
         return dd::fail(DD_ERR_INVALID, "NULL argument or unknown dtype");
     dd::Geometry g;
     dd_status st = dd::plan_geometry(p, t, &g);  // resolves an automatic choice
@@ -546,7 +400,7 @@ dd_status dd_plan_get_tiles(dd_plan_t p, dd_dtype t, dd_tiles *out) {
 }
 
 dd_status dd_plan_set_tiles(dd_plan_t p, dd_dtype t, const dd_tiles *tl) {
-    if (!p || !tl || !valid_dtype(t))
+    if (!p || !tl || !dd::valid_dtype(t))
         return dd::fail(DD_ERR_INVALID, "NULL argument or unknown dtype");
     dd::Geometry g;
     dd_status st = dd::make_geometry(p, t, *tl, &g);
