@@ -390,7 +390,9 @@ typedef struct dd_batch_s *dd_batch_t;
  * an atomic counter.  The launch (and the reset of the counter before it) is
  * captured once into a CUDA graph and replayed by later
  * dd_batch_execute calls (re-captured after dd_batch_set_io or a tile change).
- * All beams share one tile shape (dd_batch_set_tiles / dd_batch_autotune);
+ * All beams share one tile shape (dd_batch_set_tiles / dd_batch_autotune; else,
+ * for FP16/FP32, the one in which their tiles are expected to finish first,
+ * chosen anew after dd_batch_set_io);
  * with the preferred uint8 shape, beams that gain by channel groups (see
  * dd_execute) run in a second launch beside it.
  * plans[i] must outlive the batch; the batch owns its device descriptors and

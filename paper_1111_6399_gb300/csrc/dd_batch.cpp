@@ -84,6 +84,15 @@ void drop_graph(dd_batch_s *b) {
     b->prepared = false;
 }
 
+// The shape for the beams as they are bound (beams without buffers count with
+// 65536 samples).
+bool choose_tiles(dd_batch_s *b, dd_tiles *tiles) {
+    std::vector<dd::BatchLoad> load;
+    for (const BatchBeam &bb : b->beams)
+        load.push_back({bb.plan, bb.bound ? bb.nsamp_out : 65536});
+    return dd::shared_tiles(load, b->dtype, tiles);
+}
+
 // Geometry, descriptors and launch shape for the current tiles.
 dd_status prepare(dd_batch_s *b) {
     if (b->prepared)
@@ -97,18 +106,8 @@ dd_status prepare(dd_batch_s *b) {
     if (b->dev >= 0 && dev != b->dev)
         return fail(DD_ERR_INVALID, "a batch is bound to the device it was first executed on");
     b->dev = dev;
-    if (!b->tiles_set) {
-        bool found = false;
-        for (const dd_tiles &cand : dd::auto_tiles(b->dtype))
-            if (fits_all(b, cand)) {
-                b->tiles = cand;
-                found = true;
-                break;
-            }
-        if (!found)
-            return fail(DD_ERR_INVALID, "no tile shape fits every beam of the batch");
-        b->tiles_set = true;
-    }
+    if (!b->tiles_set && !choose_tiles(b, &b->tiles))
+        return fail(DD_ERR_INVALID, "no tile shape fits every beam of the batch");
     const int elem = dd::elem_size(b->dtype);
     int64_t stage_max = 0;
     for (auto &bb : b->beams) {
@@ -335,16 +334,9 @@ dd_status dd_batch_get_tiles(dd_batch_t b, dd_tiles *t) {
     if (!b || !t)
         return fail(DD_ERR_INVALID, "NULL argument");
     std::lock_guard<std::mutex> lk(b->mu);
-    if (!b->tiles_set) {
-        for (const dd_tiles &cand : dd::auto_tiles(b->dtype))
-            if (fits_all(b, cand)) {
-                b->tiles = cand;
-                b->tiles_set = true;
-                break;
-            }
-        if (!b->tiles_set)
-            return fail(DD_ERR_INVALID, "no tile shape fits every beam of the batch");
-    }
+    // (A prepared batch has its shape; else the one that its next execution takes.)
+    if (!b->tiles_set && !b->prepared && !choose_tiles(b, &b->tiles))
+        return fail(DD_ERR_INVALID, "no tile shape fits every beam of the batch");
     *t = b->tiles;
     return DD_OK;
 }

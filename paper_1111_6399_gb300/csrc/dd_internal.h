@@ -220,6 +220,27 @@ double execution_time(dd_plan_s *p, dd_dtype t, int64_t nsamp_out);
 double direct_time_us(dd_plan_s *p, dd_dtype t, const dd_tiles &tl, int64_t nsamp_out, int sms);
 double direct_tile_us(dd_plan_s *p, dd_dtype t, const dd_tiles &tl);
 
+// Time to finish tiles that are handed out in order, each to the first free SM.
+class Makespan {
+  public:
+    explicit Makespan(int sms) : sms_(std::max(1, sms)) { free_[0.0] = sms_; }
+    void run(int64_t tiles, double us);
+    double end() const { return end_; }
+
+  private:
+    int sms_;
+    double end_ = 0;
+    std::map<double, int> free_;  // when free -> SMs
+};
+
+// The tile shape that a batch or a server takes for its beams while none has
+// been set; false: no shape fits all of them.
+struct BatchLoad {
+    dd_plan_s *plan;
+    int64_t nsamp_out;
+};
+bool shared_tiles(const std::vector<BatchLoad> &beams, dd_dtype t, dd_tiles *out);
+
 // Launch shape for the DMs of the last, partly filled DM tile of geometry g,
 // run as a launch of their own (see dd_plan.cpp); cached per tile shape.
 dd_status tail_geometry(dd_plan_s *p, dd_dtype t, const Geometry &g, bool *found,

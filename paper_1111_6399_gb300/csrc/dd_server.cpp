@@ -250,19 +250,17 @@ dd_status start(dd_server_s *v) {
     cudaDeviceGetAttribute(&v->nsm, cudaDevAttrMultiProcessorCount, v->dev);
     if (v->nsm < 1)
         v->nsm = 1;
-    bool found = false;
-    for (const dd_tiles &cand : dd::auto_tiles(v->dtype)) {
-        bool ok = true;
-        for (auto &b : v->beams)
-            ok = ok && dd::make_geometry(b.plan, v->dtype, cand, &b.g) == DD_OK;
-        if (ok) {
-            v->tiles = cand;
-            found = true;
-            break;
-        }
-    }
-    if (!found)
+    // The shape for a launch that holds a block of every beam.
+    std::vector<dd::BatchLoad> load;
+    for (const SrvBeam &b : v->beams)
+        load.push_back({b.plan, b.B});
+    if (!dd::shared_tiles(load, v->dtype, &v->tiles))
         return fail(DD_ERR_INVALID, "no tile shape fits every beam of the server");
+    for (auto &b : v->beams) {
+        const dd_status st = dd::make_geometry(b.plan, v->dtype, v->tiles, &b.g);
+        if (st != DD_OK)
+            return st;
+    }
     int64_t nchan_max = 0, ndm_max = 0, B_max = 0, SB_max = 0;
     int64_t stage_max = 0;
     int64_t tails = 0;

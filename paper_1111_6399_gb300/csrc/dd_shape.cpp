@@ -8,6 +8,11 @@
 // three stages.  With the preferred shape alone, 64 channels x 64 DMs x 8192
 // samples took 29 us (16 CTAs on 152 SMs) against 15, and 512 x 200 x 8192 took
 // 153 against 71.
+//
+// A batch or a server has one shape for all its beams: the one in which their
+// tiles, largest beams first, are expected to keep the SMs busy for the least
+// time.  Eight FP32 beams of 1024 channels x 24 DMs x 16384 samples took 888 us
+// in 48-DM tiles, half of them padding, against 575 in 24-DM tiles.
 #include <cuda_runtime_api.h>
 
 #include <algorithm>
@@ -188,6 +193,95 @@ int fastest_shape(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, int sms, double *
 }
 
 }  // namespace
+
+void Makespan::run(int64_t tiles, double us) {
+    if (tiles > 4 * (int64_t)sms_) {  // whole rounds at once
+        const int64_t rounds = tiles / sms_ - 2;
+        std::map<double, int> later;
+        for (const auto &f : free_)
+            later[f.first + (double)rounds * us] += f.second;
+        free_.swap(later);
+        tiles -= rounds * sms_;
+    }
+    while (tiles > 0) {
+        const auto first = free_.begin();
+        const double at = first->first;
+        const int n = (int)std::min<int64_t>(tiles, first->second);
+        if ((first->second -= n) == 0)
+            free_.erase(first);
+        free_[at + us] += n;
+        end_ = std::max(end_, at + us);
+        tiles -= n;
+    }
+}
+
+namespace {
+
+bool fits_every(const std::vector<BatchLoad> &beams, dd_dtype t, const dd_tiles &tl) {
+    Geometry g;
+    for (const BatchLoad &b : beams)
+        if (make_geometry(b.plan, t, tl, &g) != DD_OK)
+            return false;
+    return true;
+}
+
+// The listed shape in which one persistent launch (a CTA per SM) over the
+// beams, largest channel counts first, is expected to finish first (-1: none
+// fits all of them).
+int fastest_shared_shape(std::vector<BatchLoad> beams, dd_dtype t, int sms) {
+    const std::vector<ShapeCost> &shapes = shape_costs(t);
+    std::stable_sort(beams.begin(), beams.end(), [](const BatchLoad &x, const BatchLoad &y) {
+        return x.plan->nchan > y.plan->nchan;
+    });
+    // All beams share the ring of the widest windows.
+    std::vector<ShapeFit> fits(shapes.size(), ShapeFit{4, 1});
+    for (const BatchLoad &b : beams) {
+        std::lock_guard<std::mutex> lk(b.plan->mu);
+        const std::vector<ShapeFit> &f = shape_fits(b.plan, t);
+        for (size_t i = 0; i < fits.size(); ++i)
+            fits[i].stages = std::min(fits[i].stages, f[i].stages);
+    }
+    int best = -1;
+    double least = 0;
+    for (int i = 0; i < (int)shapes.size(); ++i) {
+        if (fits[i].stages == 0 || (shapes[i].wide && fits[0].stages >= 3))
+            continue;
+        const Geometry g = tile_geometry(t, shapes[i].tiles);
+        Makespan m(sms);
+        for (const BatchLoad &b : beams)
+            m.run((int64_t)((b.plan->ndm + g.dm_cta - 1) / g.dm_cta) *
+                      ((b.nsamp_out + g.t_cta - 1) / g.t_cta),
+                  tile_us(t, shapes[i], fits[i], b.plan->nchan, 1));
+        const double us = m.end() * (i > 0 ? 1.02 : 1.0);
+        if (best < 0 || us < least) {
+            best = i;
+            least = us;
+        }
+    }
+    return best;
+}
+
+}  // namespace
+
+bool shared_tiles(const std::vector<BatchLoad> &beams, dd_dtype t, dd_tiles *out) {
+    int dev = 0;
+    const int sms = cudaGetDevice(&dev) == cudaSuccess ? sm_count(dev) : 0;
+    // (uint8 keeps the preferred shape: beams of few DMs gain by the channel
+    // groups that stand beside it.)
+    if (t != DD_U8 && sms > 0) {
+        const int best = fastest_shared_shape(beams, t, sms);
+        if (best >= 0 && fits_every(beams, t, shape_costs(t)[(size_t)best].tiles)) {
+            *out = shape_costs(t)[(size_t)best].tiles;
+            return true;
+        }
+    }
+    for (const dd_tiles &cand : auto_tiles(t))
+        if (fits_every(beams, t, cand)) {
+            *out = cand;
+            return true;
+        }
+    return false;
+}
 
 double direct_time_us(dd_plan_s *p, dd_dtype t, const dd_tiles &tl, int64_t nsamp_out, int sms) {
     const int i = place_of(t, tl);
