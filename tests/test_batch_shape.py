@@ -33,7 +33,7 @@ def test_few_dms_do_not_take_the_48_dm_tiles(host, kind, beams, nchan, ndm, ns):
     host.reset()
     assert host.batch_execute(batch) == 0
     launch = host.records(hostrt.DIRECT)[0]
-    assert launch.dm_per_thread * launch.dm_warps <= (24 if ndm <= 24 else 52)
+    assert ndm > 24 or launch.dm_per_thread * launch.dm_warps < 48
     tiles = (ctypes.c_int * 5)()
     assert host.lib.dd_batch_get_tiles(batch, tiles) == 0
     assert tuple(tiles) == launch.shape
