@@ -167,25 +167,31 @@ dd_status prepare(dd_batch_s *b) {
         d.pad = 0;
         tile0 += bb.ntiles;
     }
-    if (!b->d_beams) {
-        if (cudaMalloc((void **)&b->d_beams, sizeof(dd::BeamArgs) * b->beams.size()) != cudaSuccess ||
-            cudaMalloc((void **)&b->d_gbeams, sizeof(dd::GroupBeam) * b->beams.size()) != cudaSuccess ||
-            cudaMalloc((void **)&b->d_counter, sizeof(int)) != cudaSuccess ||
-            cudaMalloc((void **)&b->d_status, sizeof(int)) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(DD_ERR_NOMEM, "batch descriptor allocation failed");
-        }
-        cudaMemset(b->d_status, 0, sizeof(int));
+    // Each on its own: what an earlier call could not have is asked for again.
+    auto have = [](auto **p, size_t bytes) {
+        return *p || cudaMalloc((void **)p, bytes) == cudaSuccess;
+    };
+    const bool fresh = !b->d_status;
+    if (!have(&b->d_beams, sizeof(dd::BeamArgs) * b->beams.size()) ||
+        !have(&b->d_gbeams, sizeof(dd::GroupBeam) * b->beams.size()) ||
+        !have(&b->d_counter, sizeof(int)) || !have(&b->d_status, sizeof(int))) {
+        cudaGetLastError();
+        return fail(DD_ERR_NOMEM, "batch descriptor allocation failed");
     }
+    if (fresh)
+        cudaMemset(b->d_status, 0, sizeof(int));
     if (cudaMemcpy(b->d_beams, desc.data(), sizeof(dd::BeamArgs) * desc.size(),
                    cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(b->d_gbeams, gdesc.data(), sizeof(dd::GroupBeam) * gdesc.size(),
                    cudaMemcpyHostToDevice) != cudaSuccess)
         return fail(DD_ERR_CUDA, "batch descriptor upload failed");
-    if (!gdesc.empty() && !desc.empty() && !b->side &&
-        (cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking) != cudaSuccess ||
-         cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess ||
-         cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming) != cudaSuccess))
+    auto event = [](cudaEvent_t *e) {
+        return *e || cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+    };
+    if (!gdesc.empty() && !desc.empty() &&
+        ((!b->side &&
+          cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking) != cudaSuccess) ||
+         !event(&b->fork) || !event(&b->join)))
         return fail(DD_ERR_CUDA, "batch stream creation failed");
     if (tile0 > 0x7fffffffLL || gtile0 > 0x7fffffffLL)
         return fail(DD_ERR_INVALID, "too many tiles in one batch");
