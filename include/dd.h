@@ -162,12 +162,15 @@ dd_status dd_autotune(dd_plan_t plan, const void *in, dd_dtype dtype, int64_t in
  * recorded on `stream` before the call's work, and `stream` waits for its
  * completion, so every later operation on `stream` sees the whole plane.
  * uint8 beams whose shape has not been set (or is the default: 4 DMs x 8 words
- * per thread, 12 DM warps, 8-channel stages) and whose neighbouring channels' shifts differ little
- * run in a kernel of its own tiles (64 DMs x 1024 samples) that sums groups of
- * channels once per shift pattern, where a count of tile rounds says it
- * finishes earlier; the sums are the same.  Its table (2.5 KB per 64 DMs and 8
- * channels) is built on the first such call, outside `stream`, and held with
- * the plan; without memory for it the direct kernel runs. */
+ * per thread, 12 DM warps, 8-channel stages) and whose neighbouring channels'
+ * shifts differ little run in a kernel of its own tiles (64 DMs x 1024 samples)
+ * that sums groups of 4 (or 3) channels once per shift pattern, where a count of
+ * tile rounds says it finishes earlier; the sums are the same.  It reads a table
+ * (2 KB per 64 DMs and 8, or 6, channels) that is held with the plan.  The call
+ * that first would use it builds it, outside `stream`: before its launch if the
+ * call gains more by it than it costs, or is captured into a graph, else behind
+ * the direct kernel, for the calls that come once it is complete.  Without
+ * memory for it the direct kernel runs. */
 dd_status dd_execute(dd_plan_t plan, const void *in, dd_dtype dtype, int64_t in_pitch,
                      int64_t nsamp_in, float *out, int64_t out_pitch, int64_t nsamp_out,
                      void *stream);
@@ -394,7 +397,10 @@ typedef struct dd_batch_s *dd_batch_t;
  * for FP16/FP32, the one in which their tiles are expected to finish first,
  * chosen anew after dd_batch_set_io);
  * with the preferred uint8 shape, beams that gain by channel groups (see
- * dd_execute) run in a second launch beside it.
+ * dd_execute) run in a second launch beside it, if the batch as a whole is
+ * expected to finish earlier.  Tables that they lack are built before the first
+ * execution if that gains more than they cost, else behind it: the graph is then
+ * captured by the first execution that finds them complete.
  * plans[i] must outlive the batch; the batch owns its device descriptors and
  * counters. */
 dd_status dd_batch_create(const dd_plan_t *plans, int nbeams, dd_dtype dtype,

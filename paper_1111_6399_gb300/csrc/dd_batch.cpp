@@ -15,6 +15,7 @@
 #include <cuda_runtime_api.h>
 
 #include <algorithm>
+#include <cstring>
 #include <mutex>
 #include <numeric>
 #include <string>
@@ -60,6 +61,11 @@ struct dd_batch_s {
     int threads = 0, smem = 0;
     int64_t total_tiles = 0;
     bool prepared = false;
+    int slot = 0;               // of the descriptors in use (two, so that a launch
+                                // in flight keeps its own)
+    std::vector<int> order;     // beams in launch order
+    bool unsampled = false;     // whether beams gain by groups is to be seen behind the launch
+    std::vector<int> tables;    // beams whose tables the next preparation waits for
     cudaStream_t capture = nullptr;
     cudaGraphExec_t exec = nullptr;
     std::mutex mu;
@@ -82,6 +88,8 @@ void drop_graph(dd_batch_s *b) {
         b->exec = nullptr;
     }
     b->prepared = false;
+    b->unsampled = false;
+    b->tables.clear();
 }
 
 // The shape for the beams as they are bound (beams without buffers count with
@@ -93,8 +101,60 @@ bool choose_tiles(dd_batch_s *b, dd_tiles *tiles) {
     return dd::shared_tiles(load, b->dtype, tiles);
 }
 
-// Geometry, descriptors and launch shape for the current tiles.
-dd_status prepare(dd_batch_s *b) {
+// Beams (in launch order) that run grouped, if the batch is expected to finish
+// earlier by it: beside the persistent launch of the others, their tiles take
+// the SMs that its CTAs leave.  A beam is a candidate if its tiles are a smaller
+// share of the SMs' time; the times compared are those of the whole batch (3
+// beams of 1024 channels x 100 DMs x 16384 samples: 144 tiles, one round of
+// 306 us; grouped, 96 longer ones, 383 us).
+//
+// Finding that out samples every plan's patterns, some 30 us of host work each
+// once.  Unless `all`, a batch of less than 400 us per plan to be sampled leaves
+// it to be done behind its launch (b->unsampled).
+std::vector<int> grouped_beams(dd_batch_s *b, bool all, double *gain_us) {
+    const dd_tiles pref = dd::default_tiles(DD_U8);
+    const int sms = dd::sm_count(b->dev);
+    std::vector<int> grouped;
+    b->unsampled = false;
+    if (b->dtype != DD_U8 || sms <= 0 || std::memcmp(&pref, &b->tiles, sizeof(pref)) != 0)
+        return grouped;
+    dd::Makespan direct(sms), mixed(sms);
+    int unsampled = 0;
+    for (int i : b->order) {
+        BatchBeam &bb = b->beams[i];
+        direct.run(bb.ntiles, dd::direct_tile_us(bb.plan, DD_U8, b->tiles));
+        unsampled += dd::group_sampled(bb.plan, b->dev) ? 0 : 1;
+    }
+    if (!all && direct.end() < 400.0 * unsampled) {
+        b->unsampled = true;
+        return grouped;
+    }
+    std::vector<dd::GroupEstimate> est;
+    for (int i : b->order) {
+        BatchBeam &bb = b->beams[i];
+        const double us = dd::direct_tile_us(bb.plan, DD_U8, b->tiles);
+        dd::GroupEstimate e;
+        if (us > 0 && dd::group_estimate(bb.plan, b->dev, bb.nsamp_out, &e) &&
+            (double)e.tiles * e.tile_us <= dd::kGroupGain * (double)bb.ntiles * us) {
+            grouped.push_back(i);
+            est.push_back(e);
+        } else {
+            mixed.run(bb.ntiles, us);
+        }
+    }
+    for (const dd::GroupEstimate &e : est)
+        mixed.run(e.tiles, e.tile_us);
+    *gain_us = direct.end() - mixed.end();
+    if (mixed.end() > dd::kGroupGain * direct.end())
+        grouped.clear();
+    return grouped;
+}
+
+// Geometry, descriptors and launch shape for the current tiles.  Tables that
+// some beams would need and do not have are built first if `now` or if this
+// execution gains more than they cost; else all beams run directly and
+// b->tables names the beams whose tables are to be started behind the launch.
+dd_status prepare(dd_batch_s *b, bool now) {
     if (b->prepared)
         return DD_OK;
     for (size_t i = 0; i < b->beams.size(); ++i)
@@ -127,26 +187,45 @@ dd_status prepare(dd_batch_s *b) {
         return fail(DD_ERR_INVALID, "batch tile shape does not fit shared memory");
 
     // Scheduling order: larger per-tile cost (channels) first.
-    std::vector<int> order(b->beams.size());
+    std::vector<int> &order = b->order;
+    order.resize(b->beams.size());
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
         return b->beams[x].plan->nchan > b->beams[y].plan->nchan;
     });
+    std::vector<dd::DevTables *> tables(b->beams.size());
+    for (size_t i = 0; i < b->beams.size(); ++i) {
+        const dd_status st = dd::device_tables(b->beams[i].plan, &tables[i]);
+        if (st != DD_OK)
+            return st;
+    }
+    const int nsm = dd::sm_count(dev);
+    double gain = 0;
+    std::vector<int> grouped = grouped_beams(b, now, &gain), missing;
+    std::vector<dd::GroupShape> shapes(b->beams.size());
+    for (int i : grouped)
+        if (!dd::group_ready(b->beams[i].plan, dev, *tables[i], false, &shapes[i]))
+            missing.push_back(i);
+    b->tables.clear();
+    if (!missing.empty() && !now && gain <= dd::kGroupTableUs * (double)missing.size()) {
+        grouped.clear();
+        b->tables = missing;
+    } else {
+        for (int i : missing)  // all of them under way before the first is waited for
+            dd::group_start(b->beams[i].plan, dev, *tables[i]);
+    }
     std::vector<dd::BeamArgs> desc;
     std::vector<dd::GroupBeam> gdesc;
     int64_t tile0 = 0, gtile0 = 0;
-    for (size_t k = 0; k < order.size(); ++k) {
-        BatchBeam &bb = b->beams[order[k]];
-        dd::DevTables *dt = nullptr;
-        dd_status st = dd::device_tables(bb.plan, &dt);
-        if (st != DD_OK)
-            return st;
-        dd::GroupShape gs;
-        if (dd::group_shape(bb.plan, b->dtype, bb.g, *dt, bb.nsamp_out, false, &gs)) {
-            gdesc.push_back(dd::group_beam(gs, *dt, bb.in, bb.in_pitch, bb.nsamp_in, bb.out,
-                                           bb.out_pitch, bb.nsamp_out));
+    for (int i : order) {
+        BatchBeam &bb = b->beams[i];
+        const dd::DevTables *dt = tables[i];
+        if (std::find(grouped.begin(), grouped.end(), i) != grouped.end() &&
+            dd::group_ready(bb.plan, dev, *dt, true, &shapes[i])) {
+            gdesc.push_back(dd::group_beam(shapes[i], *dt, bb.in, bb.in_pitch, bb.nsamp_in,
+                                           bb.out, bb.out_pitch, bb.nsamp_out));
             gdesc.back().tile_begin = gtile0;
-            gtile0 += dd::group_tiles(gs, bb.nsamp_out);
+            gtile0 += dd::group_tiles(shapes[i], bb.nsamp_out);
             continue;
         }
         desc.emplace_back();
@@ -171,19 +250,27 @@ dd_status prepare(dd_batch_s *b) {
     auto have = [](auto **p, size_t bytes) {
         return *p || cudaMalloc((void **)p, bytes) == cudaSuccess;
     };
+    const size_t n = b->beams.size();
     const bool fresh = !b->d_status;
-    if (!have(&b->d_beams, sizeof(dd::BeamArgs) * b->beams.size()) ||
-        !have(&b->d_gbeams, sizeof(dd::GroupBeam) * b->beams.size()) ||
+    if (!have(&b->d_beams, 2 * sizeof(dd::BeamArgs) * n) ||
+        !have(&b->d_gbeams, 2 * sizeof(dd::GroupBeam) * n) ||
         !have(&b->d_counter, sizeof(int)) || !have(&b->d_status, sizeof(int))) {
         cudaGetLastError();
         return fail(DD_ERR_NOMEM, "batch descriptor allocation failed");
     }
     if (fresh)
         cudaMemset(b->d_status, 0, sizeof(int));
-    if (cudaMemcpy(b->d_beams, desc.data(), sizeof(dd::BeamArgs) * desc.size(),
-                   cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(b->d_gbeams, gdesc.data(), sizeof(dd::GroupBeam) * gdesc.size(),
-                   cudaMemcpyHostToDevice) != cudaSuccess)
+    if (!b->capture &&
+        cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking) != cudaSuccess)
+        return fail(DD_ERR_CUDA, "capture stream creation failed");
+    b->slot ^= 1;
+    dd::BeamArgs *d_beams = b->d_beams + (size_t)b->slot * n;
+    dd::GroupBeam *d_gbeams = b->d_gbeams + (size_t)b->slot * n;
+    if (cudaMemcpyAsync(d_beams, desc.data(), sizeof(dd::BeamArgs) * desc.size(),
+                        cudaMemcpyHostToDevice, b->capture) != cudaSuccess ||
+        cudaMemcpyAsync(d_gbeams, gdesc.data(), sizeof(dd::GroupBeam) * gdesc.size(),
+                        cudaMemcpyHostToDevice, b->capture) != cudaSuccess ||
+        cudaStreamSynchronize(b->capture) != cudaSuccess)
         return fail(DD_ERR_CUDA, "batch descriptor upload failed");
     auto event = [](cudaEvent_t *e) {
         return *e || cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
@@ -195,12 +282,10 @@ dd_status prepare(dd_batch_s *b) {
         return fail(DD_ERR_CUDA, "batch stream creation failed");
     if (tile0 > 0x7fffffffLL || gtile0 > 0x7fffffffLL)
         return fail(DD_ERR_INVALID, "too many tiles in one batch");
-    int nsm = 0;
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     b->total_tiles = tile0;
     b->ggrid = (unsigned)gtile0;
     b->gargs = dd::GroupArgs{};
-    b->gargs.beams = b->d_gbeams;
+    b->gargs.beams = d_gbeams;
     b->gargs.nbeams = (int)gdesc.size();
     b->gargs.status = b->d_status;
     b->grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(tile0, nsm > 0 ? nsm : 1));
@@ -208,7 +293,7 @@ dd_status prepare(dd_batch_s *b) {
     b->smem = (int)smem_for(nst);
     dd::KArgs &a = b->args;
     a = dd::KArgs{};
-    a.beams = b->d_beams;
+    a.beams = d_beams;
     a.nbeams = (int)desc.size();
     a.total_tiles = tile0;
     a.tile_counter = b->d_counter;
@@ -223,6 +308,29 @@ dd_status prepare(dd_batch_s *b) {
     a.status = b->d_status;
     b->prepared = true;
     return DD_OK;
+}
+
+// Between executions: start the tables that the next preparation is to use;
+// once all of them have come (or failed) the batch is to be prepared anew.
+void look_after_tables(dd_batch_s *b) {
+    if (b->unsampled) {
+        double gain = 0;
+        b->tables = grouped_beams(b, true, &gain);
+    }
+    if (b->tables.empty())
+        return;
+    bool waiting = false;
+    for (int i : b->tables) {
+        BatchBeam &bb = b->beams[i];
+        dd::DevTables *dt = nullptr;
+        dd::GroupEstimate e;
+        if (dd::device_tables(bb.plan, &dt) != DD_OK)
+            continue;
+        dd::group_start(bb.plan, b->dev, *dt);
+        waiting |= dd::group_estimate(bb.plan, b->dev, bb.nsamp_out, &e) && !e.ready;
+    }
+    if (!waiting)
+        drop_graph(b);
 }
 
 // The tile counter reset and the persistent launch of the direct beams; the
@@ -370,15 +478,16 @@ dd_status dd_batch_execute(dd_batch_t b, void *stream) {
     std::lock_guard<std::mutex> lk(b->mu);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (!b->exec) {
-        dd_status st = prepare(b);
+        look_after_tables(b);
+        dd_status st = prepare(b, false);
         if (st != DD_OK)
             return st;
         // One eager run first: it sets the kernel attributes outside any capture.
         if ((st = enqueue(b, s)) != DD_OK)
             return st;
-        if (!b->capture &&
-            cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking) != cudaSuccess)
-            return fail(DD_ERR_CUDA, "capture stream creation failed");
+        look_after_tables(b);
+        if (!b->prepared || !b->tables.empty())
+            return DD_OK;  // a later execution has the graph
         cudaGraph_t graph = nullptr;
         if (cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
             return fail(DD_ERR_CUDA, "stream capture failed to start");
@@ -452,7 +561,7 @@ dd_status dd_batch_autotune(dd_batch_t b, void *stream, int reps, dd_tune_result
             drop_graph(b);
             b->tiles = c;
             b->tiles_set = true;
-            if ((st = prepare(b)) != DD_OK)
+            if ((st = prepare(b, true)) != DD_OK)
                 break;
             if ((st = enqueue(b, s)) != DD_OK)  // warm-up
                 break;

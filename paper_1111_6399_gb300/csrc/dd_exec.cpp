@@ -9,6 +9,7 @@
 #include <string>
 #include <vector>
 
+#include "dd_group.h"
 #include "dd_internal.h"
 
 namespace {
@@ -148,6 +149,10 @@ extern "C" dd_status dd_execute_host(dd_plan_t p, const void *in_host, dd_dtype 
     std::lock_guard<std::mutex> lk(ws_mu);
     HostWorkspace &ws = ws_by_dev[dev];
 
+    dd::Geometry whole;
+    if ((st = dd::execution_geometry(p, dtype, nsamp_out, &whole)) != DD_OK)
+        return st;
+
     const int64_t elem = dd::elem_size(dtype);
     const int64_t S = p->maxshift;
     // Output blocks: short first and last blocks (the first block's input
@@ -237,6 +242,11 @@ extern "C" dd_status dd_execute_host(dd_plan_t p, const void *in_host, dd_dtype 
             e = cudaEventRecord(ws.landed[i], s);
         if (e != cudaSuccess)
             return fail(DD_ERR_CUDA, std::string("input copy: ") + cudaGetErrorString(e));
+        // A table for the blocks to come, while the first one's input is copied, if
+        // all of them together gain more by it than it costs.
+        dd::GroupShape gs;
+        if (k == 0)
+            dd::group_route(p, dtype, whole, *dt, nsamp_out, false, &gs);
         dd::Geometry g;
         if ((st = dd::execution_geometry(p, dtype, nb, &g)) != DD_OK)
             return st;
@@ -397,11 +407,13 @@ extern "C" dd_status dd_autotune(dd_plan_t p, const void *in, dd_dtype dtype, in
         float ms = -1.0f;
         if (dd::make_geometry(p, dtype, cand, &g) == DD_OK) {
             st = dd::launch_dedisperse(p, g, *dt, in, dtype, in_pitch, nsamp_in, out,
-                                           out_pitch, nsamp_out, s);  // warm-up
+                                           out_pitch, nsamp_out, s, true,
+                                           dd::Grouped::kNow);  // warm-up
             for (int r = 0; r < reps && st == DD_OK; ++r) {
                 cudaEventRecord(e0, s);
                 st = dd::launch_dedisperse(p, g, *dt, in, dtype, in_pitch, nsamp_in, out,
-                                               out_pitch, nsamp_out, s);
+                                               out_pitch, nsamp_out, s, true,
+                                               dd::Grouped::kNow);
                 cudaEventRecord(e1, s);
                 if (cudaEventSynchronize(e1) != cudaSuccess) {
                     st = fail(DD_ERR_CUDA, "autotune synchronize failed");

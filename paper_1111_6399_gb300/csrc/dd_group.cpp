@@ -17,6 +17,7 @@ struct Sample {
     double nt = 0;      // patterns of a group
     double reach = 0;   // reference shifts a pattern spans (samples)
     double spread = 0;  // reference shifts a tile spans
+    double bytes = 0;   // of the arrays of the largest group sampled
     bool fits = true;
 };
 
@@ -58,8 +59,11 @@ Sample sample_patterns(const dd_plan_s *p, int G) {
                 s_lo = std::min(s_lo, s0);
                 s_hi = std::max(s_hi, s0);
             }
+            double reach = 0;
             for (int t = 0; t < nt; ++t)
-                r.reach += hi[t] - lo[t];
+                reach += hi[t] - lo[t];
+            r.reach += reach;
+            r.bytes = std::max(r.bytes, 4.0 * (nt * kGroupTCta + reach));
             patterns += nt;
             r.spread += s_hi - s_lo;
         }
@@ -84,99 +88,189 @@ double group_clocks(const Sample &s, int G) {
 // Prologue and epilogue of a tile, clocks.
 constexpr double kTileClocks = 10000;
 constexpr double kClocksPerUs = 2070;
-// Grouped execution is taken when it is expected to gain this much: the model
-// is good to about 5 %.
-constexpr double kGain = 0.95;
+// Executions shorter than this by the direct kernel stay with it: a table costs
+// more than shorter beams gain in many.
+constexpr double kLeastUs = 100.0;
+// The patterns are sampled before an execution only if it is longer than this;
+// behind a shorter one otherwise.
+constexpr double kSampleUs = 1000.0;
+
+// The grouped form of the plan on device dev, its patterns sampled.  Caller
+// holds p->mu.
+GroupShape &shape_of(dd_plan_s *p, int dev) {
+    auto it = p->group.find(dev);
+    if (it != p->group.end())
+        return *it->second;
+    auto r = std::make_shared<GroupShape>();
+    r->ntile_d = (p->ndm + kGroupDmCta - 1) / kGroupDmCta;
+    // A staged window: the tile, its DMs' spread in the most delayed
+    // channel, the 16-byte rounding at both ends and the samples by which
+    // smallest shifts of channels disagree.
+    double spread = 0;
+    const double most = *std::max_element(p->dmshift.begin(), p->dmshift.end());
+    for (int a = 0; a < p->ndm; a += kGroupDmCta)
+        spread = std::max(
+            spread, most * ((double)p->dm_sorted[(size_t)std::min(a + kGroupDmCta, p->ndm) - 1] -
+                            (double)p->dm_sorted[(size_t)a]));
+    if (spread < 8192) {
+        r->rowcap = (kGroupTCta + (int)spread + 64 + 15) / 16 * 16;
+        for (int G : {4, 3}) {
+            const Sample s = sample_patterns(p, G);
+            // Four groups' arrays are held at once.
+            if (s.fits && kGroupRaw * group_raw_bytes(G, r->rowcap) < kGroupSmem / 2 &&
+                4.0 * s.bytes < group_array_bytes(G, r->rowcap))
+                r->sizes.push_back({G, group_clocks(s, G)});
+        }
+        std::sort(r->sizes.begin(), r->sizes.end(),
+                  [](const auto &x, const auto &y) { return x.clk < y.clk; });
+    }
+    return *p->group.emplace(dev, r).first->second;
+}
+
+void start(dd_plan_s *p, int dev, const DevTables &dt, GroupShape &r) {
+    while (!r.entries && !r.build.entries && !r.sizes.empty()) {
+        GroupPrep a{};
+        a.dmshift = dt.dmshift;
+        a.dm_sorted = dt.dm_sorted;
+        a.nchan = p->nchan;
+        a.ntile_d = r.ntile_d;
+        a.G = r.sizes[0].G;
+        a.rowcap = r.rowcap;
+        // The table is built on a stream of the library's, so a capture of
+        // the caller's stream does not see it.
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        const bool ok = start_group_table(a, dev, &r.build);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (!ok)  // no memory for it
+            r.sizes.erase(r.sizes.begin());
+    }
+}
+
+// Take in a table under way; waited for if `wait`.
+void poll(dd_plan_s *p, int dev, GroupShape &r, bool wait) {
+    if (!r.build.entries)
+        return;
+    GroupEntry *entries = r.build.entries;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const TableState st = finish_group_table(&r.build, dev, wait);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (st == TableState::kUnusable) {  // the sampled groups fitted, others do not
+        r.sizes.erase(r.sizes.begin());
+    } else if (st == TableState::kComplete) {
+        r.G = r.sizes[0].G;
+        r.npairs = ((p->nchan + r.G - 1) / r.G + 1) / 2;
+        r.entries = entries;
+        r.sizes.resize(1);
+    }
+}
+
+double tile_us(const dd_plan_s *p, const GroupShape &r) {
+    return (p->nchan * r.sizes[0].clk + kTileClocks) / kClocksPerUs;
+}
+
+// The preferred tile shape stands for the library's choice; another shape set
+// by the caller, or timed by the autotuner, runs as such.
+bool may_group(dd_dtype t, const Geometry &g) {
+    const dd_tiles pref = default_tiles(DD_U8);
+    return t == DD_U8 && (g.chosen || std::memcmp(&pref, &g.tiles, sizeof(pref)) == 0);
+}
+
+// Times of an execution alone on the device, in rounds of tiles over the SMs.
+// False: the grouped form does not gain enough.
+bool gains(dd_plan_s *p, int dev, const Geometry &g, int64_t nsamp_out, double *gain_us,
+           bool *ready) {
+    const int sms = sm_count(dev);
+    const double direct = sms > 0 ? direct_time_us(p, DD_U8, g.tiles, nsamp_out, sms) : -1.0;
+    GroupEstimate e;
+    if (direct < kLeastUs || !group_estimate(p, dev, nsamp_out, &e))
+        return false;
+    const double grouped = (double)((e.tiles + sms - 1) / sms) * e.tile_us;
+    *gain_us = direct - grouped;
+    *ready = e.ready;
+    return grouped <= kGroupGain * direct;
+}
 
 }  // namespace
 
-bool group_shape(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &dt,
-                 int64_t nsamp_out, bool alone, GroupShape *out) {
-    // The preferred tile shape stands for the library's choice; another shape
-    // set by the caller, or timed by the autotuner, runs as such.
-    const dd_tiles pref = default_tiles(DD_U8);
-    int dev = 0;
-    if (t != DD_U8 || (std::memcmp(&pref, &g.tiles, sizeof(pref)) != 0 && !g.chosen) ||
-        cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
-        return false;
-    const int sms = sm_count(dev);
-    const int64_t tiles = (nsamp_out + g.t_cta - 1) / g.t_cta * g.ntile_d;
-    if (sms <= 0)
-        return false;
-    // Time of the direct kernel: in rounds of tiles over the SMs, or, as one of
-    // many beams, its share of them (of the time of one tile's round).
-    const double direct = alone ? direct_time_us(p, t, g.tiles, nsamp_out, sms)
-                                : direct_tile_us(p, t, g.tiles) * (double)tiles / sms;
-    // A table costs a plan's first execution about 110 us (35 of them for the
-    // samples below), more than shorter beams gain in many.
-    if (direct < (alone ? 100.0 : 0.0))
-        return false;
+bool group_sampled(dd_plan_s *p, int dev) {
     std::lock_guard<std::mutex> lk(p->mu);
-    auto it = p->group.find(dev);
-    if (it == p->group.end()) {
-        auto r = std::make_shared<GroupShape>();
-        r->ntile_d = (p->ndm + kGroupDmCta - 1) / kGroupDmCta;
-        // A staged window: the tile, its DMs' spread in the most delayed
-        // channel, the 16-byte rounding at both ends and the samples by which
-        // smallest shifts of channels disagree.
-        double spread = 0;
-        const double most = *std::max_element(p->dmshift.begin(), p->dmshift.end());
-        for (int a = 0; a < p->ndm; a += kGroupDmCta)
-            spread = std::max(
-                spread,
-                most * ((double)p->dm_sorted[(size_t)std::min(a + kGroupDmCta, p->ndm) - 1] -
-                        (double)p->dm_sorted[(size_t)a]));
-        if (spread < 8192) {
-            r->rowcap = (kGroupTCta + (int)spread + 64 + 15) / 16 * 16;
-            for (int G : {4, 3}) {
-                const Sample s = sample_patterns(p, G);
-                // Four groups' arrays are held at once.
-                if (s.fits && kGroupRaw * group_raw_bytes(G, r->rowcap) < kGroupSmem / 2 &&
-                    16.0 * s.nt * (kGroupTCta + s.reach) < group_array_bytes(G, r->rowcap)) {
-                    r->sizes.push_back({G, group_clocks(s, G)});
-                }
-            }
-            std::sort(r->sizes.begin(), r->sizes.end(),
-                      [](const auto &x, const auto &y) { return x.clk < y.clk; });
-        }
-        it = p->group.emplace(dev, r).first;
+    return p->group.count(dev) != 0;
+}
+
+bool group_estimate(dd_plan_s *p, int dev, int64_t nsamp_out, GroupEstimate *e) {
+    std::lock_guard<std::mutex> lk(p->mu);
+    GroupShape &r = shape_of(p, dev);
+    poll(p, dev, r, false);
+    if (r.sizes.empty())
+        return false;
+    e->tile_us = tile_us(p, r);
+    e->tiles = group_tiles(r, nsamp_out);
+    e->ready = r.entries != nullptr;
+    return true;
+}
+
+void group_start(dd_plan_s *p, int dev, const DevTables &dt) {
+    std::lock_guard<std::mutex> lk(p->mu);
+    start(p, dev, dt, shape_of(p, dev));
+}
+
+bool group_ready(dd_plan_s *p, int dev, const DevTables &dt, bool now, GroupShape *out) {
+    std::lock_guard<std::mutex> lk(p->mu);
+    GroupShape &r = shape_of(p, dev);
+    poll(p, dev, r, now);
+    while (now && !r.entries && !r.sizes.empty()) {
+        start(p, dev, dt, r);
+        poll(p, dev, r, true);
     }
-    GroupShape &r = *it->second;
-    const double n = (double)group_tiles(r, nsamp_out) / sms;
-    while (!r.sizes.empty() &&
-           (alone ? std::ceil(n) : n) * (p->nchan * r.sizes[0].clk + kTileClocks) / kClocksPerUs <=
-               kGain * direct) {
-        if (!r.entries) {
-            GroupPrep a;
-            a.dmshift = dt.dmshift;
-            a.dm_sorted = dt.dm_sorted;
-            a.nchan = p->nchan;
-            a.ntile_d = r.ntile_d;
-            a.G = r.sizes[0].G;
-            a.rowcap = r.rowcap;
-            // The table is built on a stream of the library's, so a capture of
-            // the caller's stream does not see it.
-            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-            cudaThreadExchangeStreamCaptureMode(&mode);
-            r.entries = build_group_table(a, dev);
-            cudaThreadExchangeStreamCaptureMode(&mode);
-            if (!r.entries) {  // the sampled groups fitted, others do not
-                r.sizes.erase(r.sizes.begin());
-                continue;
-            }
-            r.G = a.G;
-            r.npairs = ((p->nchan + r.G - 1) / r.G + 1) / 2;
-            r.sizes.resize(1);
-        }
-        *out = r;
-        return true;
+    if (!r.entries)
+        return false;
+    *out = r;
+    return true;
+}
+
+GroupRoute group_route(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &dt,
+                       int64_t nsamp_out, bool now, GroupShape *out) {
+    int dev = 0;
+    if (!may_group(t, g) || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
+        return GroupRoute::kDirect;
+    if (!now && !group_sampled(p, dev)) {
+        const int sms = sm_count(dev);
+        const double direct = sms > 0 ? direct_time_us(p, t, g.tiles, nsamp_out, sms) : -1.0;
+        if (direct < kSampleUs)
+            return direct < kLeastUs ? GroupRoute::kDirect : GroupRoute::kLater;
     }
-    return false;
+    double gain = 0;
+    bool ready = false;
+    // (Again if a table turns out unusable: another group size may serve.)
+    while (gains(p, dev, g, nsamp_out, &gain, &ready)) {
+        const bool wait = now || gain > kGroupTableUs;
+        if (!ready && !wait)
+            return GroupRoute::kLater;
+        if (group_ready(p, dev, dt, wait, out))
+            return GroupRoute::kGrouped;
+    }
+    return GroupRoute::kDirect;
+}
+
+void group_later(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &dt,
+                 int64_t nsamp_out) {
+    int dev = 0;
+    double gain = 0;
+    bool ready = false;
+    if (may_group(t, g) && cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 &&
+        gains(p, dev, g, nsamp_out, &gain, &ready) && !ready)
+        group_start(p, dev, dt);
 }
 
 void group_free(dd_plan_s *p) {
     for (auto &kv : p->group) {
         cudaSetDevice(kv.first);
+        GroupEntry *building = kv.second->build.entries;
+        if (building &&
+            finish_group_table(&kv.second->build, kv.first, true) == TableState::kComplete)
+            cudaFree(building);
         cudaFree(kv.second->entries);
     }
     p->group.clear();

@@ -620,48 +620,31 @@ __global__ void __launch_bounds__(kPrepThreads) group_place_kernel(const GroupPr
 
 }  // namespace
 
-GroupEntry *build_group_table(GroupPrep a, int dev) {
-    // One library stream per device: tables are built outside the caller's
-    // streams (and their captures), and the build is complete on return.
-    static std::mutex mu;
-    static cudaStream_t streams[64] = {nullptr};
-    const size_t pairs = (size_t)a.ntile_d * (size_t)(((a.nchan + a.G - 1) / a.G + 1) / 2);
-    std::lock_guard<std::mutex> lk(mu);
-    cudaStream_t &s = streams[dev];
-    // The table, the groups' sizes, the failure flag (one allocation; freeing a
-    // second one would wait for the device).
-    const size_t table = sizeof(GroupEntry) * pairs;
-    void *mem = nullptr;
-    int failed = 1;
-    if ((s || cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess) &&
-        cudaMalloc(&mem, table + sizeof(int) * (2 * pairs + 1)) == cudaSuccess) {
-        a.entries = static_cast<GroupEntry *>(mem);
-        int *sizes = reinterpret_cast<int *>(static_cast<uint8_t *>(mem) + table);
-        a.fail = sizes + 2 * pairs;
-        const unsigned ng = 2 * (unsigned)(pairs / (size_t)a.ntile_d);
-        const dim3 grid((ng + kPrepThreads / 32 - 1) / (kPrepThreads / 32), (unsigned)a.ntile_d);
-        if (cudaMemsetAsync(a.fail, 0, sizeof(int), s) == cudaSuccess) {
-            group_prep_kernel<<<grid, kPrepThreads, 0, s>>>(a, sizes);
-            group_place_kernel<<<grid, kPrepThreads, 0, s>>>(a, sizes);
-            if (cudaGetLastError() != cudaSuccess ||
-                cudaMemcpyAsync(&failed, a.fail, sizeof(int), cudaMemcpyDeviceToHost, s) !=
-                    cudaSuccess ||
-                cudaStreamSynchronize(s) != cudaSuccess)
-                failed = 1;
-        }
-    }
-    if (failed) {
-        cudaGetLastError();
-        cudaFree(mem);
-        return nullptr;
-    }
-    return a.entries;
+namespace {
+
+// Library streams of a device: tables are built outside the caller's streams
+// (and their captures), ahead of CTAs that wait for an SM; their failure flags
+// are read on another, so that no flag waits for a later table.
+struct TableStreams {
+    cudaStream_t build = nullptr, read = nullptr;
+};
+std::mutex g_table_mu;
+TableStreams g_table_streams[64];
+
+bool table_streams(int dev, TableStreams **out) {
+    TableStreams &t = g_table_streams[dev];
+    int least = 0, greatest = 0;
+    *out = &t;
+    return (t.build || (cudaDeviceGetStreamPriorityRange(&least, &greatest) == cudaSuccess &&
+                        cudaStreamCreateWithPriority(&t.build, cudaStreamNonBlocking, greatest) ==
+                            cudaSuccess)) &&
+           (t.read ||
+            cudaStreamCreateWithFlags(&t.read, cudaStreamNonBlocking) == cudaSuccess);
 }
 
-cudaError_t launch_group(const GroupArgs &a, unsigned grid, cudaStream_t s) {
+// The attribute of group_kernel that its launches need, set once per device.
+cudaError_t configure_group_kernel(int dev) {
     static bool configured[64] = {false};
-    int dev = 0;
-    cudaGetDevice(&dev);
     bool &conf = configured[dev & 63];
     if (!conf) {
         const cudaError_t e = cudaFuncSetAttribute(
@@ -670,6 +653,77 @@ cudaError_t launch_group(const GroupArgs &a, unsigned grid, cudaStream_t s) {
             return e;
         conf = true;
     }
+    return cudaSuccess;
+}
+
+}  // namespace
+
+bool start_group_table(GroupPrep a, int dev, GroupBuild *b) {
+    const size_t pairs = (size_t)a.ntile_d * (size_t)(((a.nchan + a.G - 1) / a.G + 1) / 2);
+    std::lock_guard<std::mutex> lk(g_table_mu);
+    TableStreams *t = nullptr;
+    // The table, the groups' sizes, the failure flag (one allocation; freeing a
+    // second one would wait for the device).
+    const size_t table = sizeof(GroupEntry) * pairs;
+    void *mem = nullptr;
+    cudaEvent_t done = nullptr;
+    bool ok = table_streams(dev, &t) && configure_group_kernel(dev) == cudaSuccess &&
+              cudaEventCreateWithFlags(&done, cudaEventDisableTiming) == cudaSuccess &&
+              cudaMalloc(&mem, table + sizeof(int) * (2 * pairs + 1)) == cudaSuccess;
+    if (ok) {
+        a.entries = static_cast<GroupEntry *>(mem);
+        int *sizes = reinterpret_cast<int *>(static_cast<uint8_t *>(mem) + table);
+        a.fail = sizes + 2 * pairs;
+        const unsigned ng = 2 * (unsigned)(pairs / (size_t)a.ntile_d);
+        const dim3 grid((ng + kPrepThreads / 32 - 1) / (kPrepThreads / 32), (unsigned)a.ntile_d);
+        ok = cudaMemsetAsync(a.fail, 0, sizeof(int), t->build) == cudaSuccess;
+        if (ok) {
+            group_prep_kernel<<<grid, kPrepThreads, 0, t->build>>>(a, sizes);
+            group_place_kernel<<<grid, kPrepThreads, 0, t->build>>>(a, sizes);
+            ok = cudaGetLastError() == cudaSuccess &&
+                 cudaEventRecord(done, t->build) == cudaSuccess;
+        }
+    }
+    if (!ok) {
+        cudaGetLastError();
+        cudaFree(mem);
+        if (done)
+            cudaEventDestroy(done);
+        return false;
+    }
+    b->entries = a.entries;
+    b->fail = a.fail;
+    b->done = done;
+    return true;
+}
+
+TableState finish_group_table(GroupBuild *b, int dev, bool wait) {
+    if (!wait && cudaEventQuery(b->done) == cudaErrorNotReady) {
+        cudaGetLastError();
+        return TableState::kUnderWay;
+    }
+    int failed = 1;
+    std::lock_guard<std::mutex> lk(g_table_mu);
+    const cudaStream_t s = g_table_streams[dev].read;
+    if (cudaEventSynchronize(b->done) != cudaSuccess ||
+        cudaMemcpyAsync(&failed, b->fail, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        failed = 1;
+    cudaEventDestroy(b->done);
+    if (failed) {
+        cudaGetLastError();
+        cudaFree(b->entries);
+    }
+    *b = GroupBuild();
+    return failed ? TableState::kUnusable : TableState::kComplete;
+}
+
+cudaError_t launch_group(const GroupArgs &a, unsigned grid, cudaStream_t s) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const cudaError_t e = configure_group_kernel(dev);
+    if (e != cudaSuccess)
+        return e;
     group_kernel<<<grid, kThreads, kGroupSmem, s>>>(a);
     return cudaGetLastError();
 }

@@ -115,6 +115,13 @@ struct GroupArgs {
     int *status;
 };
 
+// A table being built on a library stream.
+struct GroupBuild {
+    GroupEntry *entries = nullptr;
+    int *fail = nullptr;  // 1 on the device when a limit does not hold (table unusable)
+    cudaEvent_t done = nullptr;
+};
+
 // Grouped execution of a plan on one device.
 struct GroupShape {
     int ntile_d = 0, rowcap = 0;
@@ -125,8 +132,9 @@ struct GroupShape {
         double clk;
     };
     std::vector<Size> sizes;
+    GroupBuild build;               // of sizes[0], under way if build.entries
     int G = 0, npairs = 0;          // of the table
-    GroupEntry *entries = nullptr;  // device table (built on first use)
+    GroupEntry *entries = nullptr;  // device table, complete
 };
 
 // Shared memory of a grouped CTA: kGroupRaw raw slots, then the array space.
@@ -146,17 +154,52 @@ struct GroupPrep {  // arguments of the table builder
     int *fail;  // set to 1 when a limit does not hold (table unusable)
 };
 
-// Build the table described by a (a.entries and a.fail are set here) on a
-// library stream of device dev; NULL, with nothing held, when a limit does
-// not hold or the device memory cannot be had.
-GroupEntry *build_group_table(GroupPrep a, int dev);
+// Start to build the table described by a (a.entries and a.fail are set here)
+// on a library stream of device dev; false, with nothing held, when the device
+// memory cannot be had.
+bool start_group_table(GroupPrep a, int dev, GroupBuild *b);
+// Its state: under way (only if not waited for), complete, or unusable (then
+// nothing is held).
+enum class TableState { kUnderWay, kComplete, kUnusable };
+TableState finish_group_table(GroupBuild *b, int dev, bool wait);
 
-// The plan's grouped form on the current device if it is expected to beat the
-// direct kernel of geometry g for nsamp_out samples, alone on the device or
-// as one of many beams (its table built on first use and kept with the plan);
-// false: use the direct kernel.
-bool group_shape(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &dt,
-                 int64_t nsamp_out, bool alone, GroupShape *out);
+// What an execution of nsamp_out samples takes in the plan's grouped form: the
+// time of a tile (microseconds), its tiles and whether the table is there.
+struct GroupEstimate {
+    double tile_us = 0;
+    int64_t tiles = 0;
+    bool ready = false;
+};
+// Whether the plan's patterns have been sampled.
+bool group_sampled(dd_plan_s *p, int dev);
+// False: no group size serves the plan.  Samples the plan's patterns on first
+// use (host work of some 30 us); polls a table under way.
+bool group_estimate(dd_plan_s *p, int dev, int64_t nsamp_out, GroupEstimate *e);
+// Start the table of the best group size if it is neither there nor under way.
+void group_start(dd_plan_s *p, int dev, const DevTables &dt);
+// The plan's grouped form, once its table is there: waited for, or started and
+// waited for (now), or left if not.
+bool group_ready(dd_plan_s *p, int dev, const DevTables &dt, bool now, GroupShape *out);
+
+// Grouped execution is taken when it is expected to gain this much: the model
+// is good to about 5 %.
+constexpr double kGroupGain = 0.95;
+// What a table costs before an execution can use it: sampling, an allocation,
+// two launches and a wait (microseconds).
+constexpr double kGroupTableUs = 200.0;
+
+// How one execution by dd_execute runs: by the direct kernel, by the direct
+// kernel with the table to be started behind it (kGroupLater: the execution
+// would gain less than the table costs it), or by the grouped kernel (*out).
+// With `now` it waits for a table in any case (graph capture: the graph keeps
+// what it captures; the autotuner).
+enum class GroupRoute { kDirect, kLater, kGrouped };
+GroupRoute group_route(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &dt,
+                       int64_t nsamp_out, bool now, GroupShape *out);
+// After a kLater launch: start the table if the plan's next execution of this
+// length would take it.
+void group_later(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &dt,
+                 int64_t nsamp_out);
 void group_free(dd_plan_s *p);
 
 GroupBeam group_beam(const GroupShape &g, const DevTables &dt, const void *in, int64_t in_pitch,

@@ -5,6 +5,7 @@
 #include <cuda_runtime_api.h>
 
 #include <algorithm>
+#include <cfloat>
 #include <cstdint>
 #include <map>
 #include <memory>
@@ -36,10 +37,8 @@ inline bool valid_dtype(dd_dtype t) { return t == DD_U8 || t == DD_F16 || t == D
 
 // The shift of a channel: one FP32 multiply, rounded to nearest even, then
 // truncated.
-inline int trunc_product(float dm, float ds) {
-    volatile float prod = dm * ds;
-    return (int)prod;
-}
+static_assert(FLT_EVAL_METHOD == 0, "float products are rounded to float");
+inline int trunc_product(float dm, float ds) { return (int)(dm * ds); }
 
 // Channels summed into 16-bit SWAR lanes before they are widened (uint8):
 // 256 * 255 = 65280 fits a 16-bit lane.
@@ -122,7 +121,7 @@ struct Geometry {
 struct GroupShape;  // dd_group.h
 
 struct ShapeFit {
-    int stages = 0;    // of the ring (0: the windows do not fit)
+    int stages = -1;   // of the ring (0: the windows do not fit, -1: not known)
     int resident = 1;  // CTAs on an SM
 };
 
@@ -143,6 +142,7 @@ struct dd_plan_s {
     bool tiles_open[3] = {true, true, true};  // executions may choose, until set
     std::map<uint64_t, dd::Geometry> geo;  // per (dtype, tiles) key
     std::vector<dd::ShapeFit> shape_fit[3];  // of the listed shapes (dd_shape.cpp), on first use
+    float most_delay = -1.0f;                // of dmshift, with the first of those
     uint32_t shape_unfit[3] = {0, 0, 0};     // shapes found not to fit, a bit each
     // Remainder-DM launch per (dtype, tiles) key: (found, geometry).
     std::map<uint64_t, std::pair<bool, dd::Geometry>> tail_geo;
@@ -250,8 +250,12 @@ dd_status tail_geometry(dd_plan_s *p, dd_dtype t, const Geometry &g, bool *found
 dd_status device_tables(dd_plan_s *p, DevTables **out);
 
 // Launch the de-dispersion of one beam on stream: the grouped kernel
-// (dd_group.cu; unless `grouped` is false) where it is expected to be faster,
-// else the direct kernel (dd_kernel_*.cu).
+// (dd_group.cu) where it is expected to be faster, else the direct kernel
+// (dd_kernel_*.cu).  kAuto: with a table that the plan does not have yet, the
+// first execution runs directly and the table is built behind it, unless this
+// execution gains more than the table costs it or a graph captures it; kNow
+// waits for the table.
+enum class Grouped { kNever, kAuto, kNow };
 // With split_tail, the DMs of a last DM tile that is at most half full run
 // as a second launch with their own tile shape, on a library stream forked
 // from and joined back into `stream`, so its CTAs fill the SMs the first
@@ -260,7 +264,7 @@ dd_status device_tables(dd_plan_s *p, DevTables **out);
 dd_status launch_dedisperse(dd_plan_s *p, const Geometry &g, const DevTables &dt,
                             const void *in, dd_dtype dtype, int64_t in_pitch, int64_t nsamp_in,
                             float *out, int64_t out_pitch, int64_t nsamp_out, void *stream,
-                            bool split_tail = true, bool grouped = true);
+                            bool split_tail = true, Grouped grouped = Grouped::kAuto);
 
 void count_launch(int n = 1);
 

@@ -162,11 +162,19 @@ dd_status launch_dedisperse_detect(dd_plan_s *p, const Geometry &g, const DevTab
 dd_status launch_dedisperse(dd_plan_s *p, const Geometry &g, const DevTables &dt, const void *in,
                             dd_dtype dtype, int64_t in_pitch, int64_t nsamp_in, float *out,
                             int64_t out_pitch, int64_t nsamp_out, void *stream,
-                            bool split_tail, bool grouped) {
+                            bool split_tail, Grouped grouped) {
     if (nsamp_out == 0)
         return DD_OK;
     GroupShape gs;
-    if (grouped && group_shape(p, dtype, g, dt, nsamp_out, true, &gs)) {
+    GroupRoute route = GroupRoute::kDirect;
+    if (grouped != Grouped::kNever && dtype == DD_U8) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) != cudaSuccess)
+            cudaGetLastError();
+        route = group_route(p, dtype, g, dt, nsamp_out,
+                            grouped == Grouped::kNow || cap != cudaStreamCaptureStatusNone, &gs);
+    }
+    if (route == GroupRoute::kGrouped) {
         cudaStream_t s = static_cast<cudaStream_t>(stream);
         const int64_t tiles = group_tiles(gs, nsamp_out);
         if (tiles > 0x7fffffffLL)
@@ -246,6 +254,8 @@ dd_status launch_dedisperse(dd_plan_s *p, const Geometry &g, const DevTables &dt
     if (g_prof_stop)
         cudaEventRecord(g_prof_stop, s);
     count_launch(split ? 2 : 1);
+    if (route == GroupRoute::kLater)
+        group_later(p, dtype, g, dt, nsamp_out);
     return DD_OK;
 }
 

@@ -145,7 +145,7 @@ extern "C" dd_status dd_execute_noalloc(dd_plan_t p, const void *in, dd_dtype dt
     dt.ndm_pad = ndm_pad;
     // One launch: the remainder-DM split needs a library stream and events.
     return dd::launch_dedisperse(p, g, dt, in, dtype, in_pitch, nsamp_in, out, out_pitch,
-                                 nsamp_out, stream, false, false);
+                                 nsamp_out, stream, false, dd::Grouped::kNever);
 }
 
 // Status of the last dd_execute_noalloc on the current device: waits for

@@ -78,47 +78,49 @@ double two_stages_us(dd_dtype t, double us) {
 // two, 61 alone).
 constexpr double kAlone = 0.88;
 
-// Ring stages (0: its windows do not fit) and CTAs on an SM of the listed
-// shapes, from the DM steps and the largest delay where those decide, else from
-// every window.  Caller holds p->mu.
-const std::vector<ShapeFit> &shape_fits(dd_plan_s *p, dd_dtype t) {
+// Ring stages (0: its windows do not fit) and CTAs on an SM of listed shape i,
+// from the DM steps and the largest delay where those decide, else from every
+// window.  Caller holds p->mu.
+const ShapeFit &shape_fit(dd_plan_s *p, dd_dtype t, int i) {
     std::vector<ShapeFit> &fits = p->shape_fit[t];
-    if (!fits.empty())
-        return fits;
-    const double most = *std::max_element(p->dmshift.begin(), p->dmshift.end());
-    for (const ShapeCost &c : shape_costs(t)) {
-        Geometry r = tile_geometry(t, c.tiles);
-        double steps = 0;
-        for (int d = 0; d < p->ndm; d += r.dm_cta)
-            steps = std::max(steps,
-                             (double)p->dm_sorted[(size_t)std::min(d + r.dm_cta, p->ndm) - 1] -
-                                 (double)p->dm_sorted[(size_t)d]);
-        // The widest window: its samples less the truncation of both shifts, and
-        // with that and the 16-byte rounding at both ends.  (Beyond 2^20 samples
-        // it fits in no shape.)
-        const int64_t spread = (int64_t)std::min(steps * most, 1048576.0);
-        auto fit = [&](int64_t widest) {
-            int64_t smem = 0;
-            ShapeFit f;
-            if (ring_layout(&r, widest, &smem)) {
-                f.stages = r.nstages;
-                f.resident = std::min(c.resident, resident_ctas(r.smem));
-            }
-            return f;
-        };
-        const int64_t samples = r.t_cta + spread;
-        ShapeFit f = fit((r.elem * (samples + 2) + 30) & ~(int64_t)15);
-        const ShapeFit most_room = fit((r.elem * std::max<int64_t>(samples - 2, 0) + 15) & ~(int64_t)15);
-        if (most_room.stages != f.stages || most_room.resident != f.resident) {
-            f = ShapeFit();
-            if (make_geometry(p, t, c.tiles, &r) == DD_OK) {
-                f.stages = r.nstages;
-                f.resident = std::min(c.resident, resident_ctas(r.smem));
-            }
+    fits.resize(shape_costs(t).size());
+    ShapeFit &f = fits[(size_t)i];
+    if (f.stages >= 0)
+        return f;
+    if (p->most_delay < 0.0f)
+        p->most_delay = *std::max_element(p->dmshift.begin(), p->dmshift.end());
+    const ShapeCost &c = shape_costs(t)[(size_t)i];
+    Geometry r = tile_geometry(t, c.tiles);
+    double steps = 0;
+    for (int d = 0; d < p->ndm; d += r.dm_cta)
+        steps = std::max(steps,
+                         (double)p->dm_sorted[(size_t)std::min(d + r.dm_cta, p->ndm) - 1] -
+                             (double)p->dm_sorted[(size_t)d]);
+    // The widest window: its samples less the truncation of both shifts, and
+    // with that and the 16-byte rounding at both ends.  (Beyond 2^20 samples it
+    // fits in no shape.)
+    const int64_t samples =
+        r.t_cta + (int64_t)std::min(steps * (double)p->most_delay, 1048576.0);
+    auto ring = [&](int64_t widest) {
+        int64_t smem = 0;
+        ShapeFit x;
+        x.stages = 0;
+        if (ring_layout(&r, widest, &smem)) {
+            x.stages = r.nstages;
+            x.resident = std::min(c.resident, resident_ctas(r.smem));
         }
-        fits.push_back(f);
+        return x;
+    };
+    f = ring((r.elem * (samples + 2) + 30) & ~(int64_t)15);
+    const ShapeFit room = ring((r.elem * std::max<int64_t>(samples - 2, 0) + 15) & ~(int64_t)15);
+    if (room.stages != f.stages || room.resident != f.resident) {
+        f.stages = 0;
+        if (make_geometry(p, t, c.tiles, &r) == DD_OK) {
+            f.stages = r.nstages;
+            f.resident = std::min(c.resident, resident_ctas(r.smem));
+        }
     }
-    return fits;
+    return f;
 }
 
 // Time of one tile with `resident` CTAs on its SM.
@@ -174,15 +176,15 @@ int place_of(dd_dtype t, const dd_tiles &tl) {
 // Caller holds p->mu.
 int fastest_shape(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, int sms, double *us) {
     const std::vector<ShapeCost> &shapes = shape_costs(t);
-    const std::vector<ShapeFit> &fits = shape_fits(p, t);
+    const bool narrow = shape_fit(p, t, 0).stages >= 3;
     int best = -1;
     for (int i = 0; i < (int)shapes.size(); ++i) {
-        if (fits[i].stages == 0 || (p->shape_unfit[t] >> i & 1u) ||
-            (shapes[i].wide && fits[0].stages >= 3))
+        if ((shapes[i].wide && narrow) || (p->shape_unfit[t] >> i & 1u) ||
+            shape_fit(p, t, i).stages == 0)
             continue;
         // (2 % in favour of the preferred shape, the first.)
         const double u =
-            shape_time_us(t, shapes[i], fits[i], p->nchan, p->ndm, nsamp_out, sms) *
+            shape_time_us(t, shapes[i], shape_fit(p, t, i), p->nchan, p->ndm, nsamp_out, sms) *
             (i > 0 ? 1.02 : 1.0);
         if (best < 0 || u < *us) {
             best = i;
@@ -235,12 +237,13 @@ int fastest_shared_shape(std::vector<BatchLoad> beams, dd_dtype t, int sms) {
     });
     // All beams share the ring of the widest windows.
     std::vector<ShapeFit> fits(shapes.size(), ShapeFit{4, 1});
-    for (const BatchLoad &b : beams) {
-        std::lock_guard<std::mutex> lk(b.plan->mu);
-        const std::vector<ShapeFit> &f = shape_fits(b.plan, t);
-        for (size_t i = 0; i < fits.size(); ++i)
-            fits[i].stages = std::min(fits[i].stages, f[i].stages);
-    }
+    for (size_t i = 0; i < fits.size(); ++i)
+        for (const BatchLoad &b : beams) {
+            if (shapes[i].wide && fits[0].stages >= 3)
+                break;
+            std::lock_guard<std::mutex> lk(b.plan->mu);
+            fits[i].stages = std::min(fits[i].stages, shape_fit(b.plan, t, (int)i).stages);
+        }
     int best = -1;
     double least = 0;
     for (int i = 0; i < (int)shapes.size(); ++i) {
@@ -286,18 +289,18 @@ bool shared_tiles(const std::vector<BatchLoad> &beams, dd_dtype t, dd_tiles *out
 double direct_time_us(dd_plan_s *p, dd_dtype t, const dd_tiles &tl, int64_t nsamp_out, int sms) {
     const int i = place_of(t, tl);
     std::lock_guard<std::mutex> lk(p->mu);
-    if (i < 0 || shape_fits(p, t)[i].stages == 0)
+    if (i < 0 || shape_fit(p, t, i).stages == 0)
         return -1.0;
-    return shape_time_us(t, shape_costs(t)[i], shape_fits(p, t)[i], p->nchan, p->ndm, nsamp_out,
-                         sms);
+    return shape_time_us(t, shape_costs(t)[(size_t)i], shape_fit(p, t, i), p->nchan, p->ndm,
+                         nsamp_out, sms);
 }
 
 double direct_tile_us(dd_plan_s *p, dd_dtype t, const dd_tiles &tl) {
     const int i = place_of(t, tl);
     std::lock_guard<std::mutex> lk(p->mu);
-    if (i < 0 || shape_fits(p, t)[i].stages == 0)
+    if (i < 0 || shape_fit(p, t, i).stages == 0)
         return -1.0;
-    return tile_us(t, shape_costs(t)[i], shape_fits(p, t)[i], p->nchan, 1);
+    return tile_us(t, shape_costs(t)[(size_t)i], shape_fit(p, t, i), p->nchan, 1);
 }
 
 dd_status execution_geometry(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, Geometry *g) {

@@ -17,7 +17,7 @@
 namespace {
 
 struct Record {
-    int kind;      // 0 direct launch, 1 grouped launch, 2 group table, 3 host-to-device copy
+    int kind;      // 0 direct launch, 1 grouped launch, 2 group table started, 3 host-to-device copy
     int dtype;     // bytes of a sample
     int dm_per_thread, dm_warps, time_warps, chan_per_stage, words;
     int beams;
@@ -29,7 +29,8 @@ struct Record {
 std::mutex mu;
 std::vector<Record> records;
 int fail_malloc = 0;  // the n-th cudaMalloc from now fails
-int table_ok = 1;
+int table_ok = 1;     // tables turn out usable
+int tables_done = 1;  // tables under way are complete when asked for
 bool capturing = false;
 int sms = 152;
 long long allocations = 0;
@@ -66,9 +67,14 @@ void fake_reset(void) {
     records.clear();
     fail_malloc = 0;
     table_ok = 1;
+    tables_done = 1;
 }
 void fake_fail_malloc(int n) { fail_malloc = n; }
-void fake_table_ok(int ok) { table_ok = ok; }
+void fake_tables(int ok, int done) {
+    table_ok = ok;
+    tables_done = done;
+}
+void fake_capturing(int on) { capturing = on != 0; }
 void fake_sms(int n) { sms = n; }
 long long fake_allocations(void) { return allocations; }
 int fake_records(Record *out, int max) {
@@ -191,15 +197,24 @@ cudaError_t launch_group(const GroupArgs &a, unsigned grid, cudaStream_t) {
     record(r);
     return grid > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
-GroupEntry *build_group_table(GroupPrep a, int) {
+bool start_group_table(GroupPrep a, int, GroupBuild *b) {
     Record r{};
     r.kind = 2;
     r.beams = a.G;
     record(r);
     void *p = nullptr;
-    if (!table_ok || cudaMalloc(&p, sizeof(GroupEntry)) != cudaSuccess)
-        return nullptr;
-    return static_cast<GroupEntry *>(p);
+    if (cudaMalloc(&p, sizeof(GroupEntry)) != cudaSuccess)
+        return false;
+    b->entries = static_cast<GroupEntry *>(p);
+    return true;
+}
+TableState finish_group_table(GroupBuild *b, int, bool wait) {
+    if (!wait && !tables_done)
+        return TableState::kUnderWay;
+    if (!table_ok)
+        cudaFree(b->entries);
+    *b = GroupBuild();
+    return table_ok ? TableState::kComplete : TableState::kUnusable;
 }
 dd_status detect_begin(int, int, double *, double *, double *, cudaStream_t) { return DD_OK; }
 dd_status detect_finalize_int(int, int64_t, int, double *, double *, double *, int64_t *,
