@@ -703,8 +703,11 @@ TableState finish_group_table(GroupBuild *b, int dev, bool wait) {
         return TableState::kUnderWay;
     }
     int failed = 1;
-    std::lock_guard<std::mutex> lk(g_table_mu);
-    const cudaStream_t s = g_table_streams[dev].read;
+    cudaStream_t s = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(g_table_mu);
+        s = g_table_streams[dev].read;
+    }
     if (cudaEventSynchronize(b->done) != cudaSuccess ||
         cudaMemcpyAsync(&failed, b->fail, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
