@@ -118,6 +118,12 @@ dd_status dd_plan_dmshift(dd_plan_t plan, float *host_out);
  * tile rounds expects to finish earlier. */
 dd_status dd_plan_get_tiles(dd_plan_t plan, dd_dtype dtype, dd_tiles *tiles_out);
 
+/* The kernel that dd_execute would now run nsamp_out uint8 samples in on the
+ * current device: channels per group (4 or 3) of the channel-group kernel, or 0
+ * for the direct kernel, as while the plan's table is not complete (see
+ * dd_execute).  Builds nothing. */
+int dd_plan_groups(dd_plan_t plan, int64_t nsamp_out);
+
 /* Override the tile shape for dtype (validated: shared-memory fit, supported
  * dm_per_thread).  Not thread-safe against concurrent executions of the plan. */
 dd_status dd_plan_set_tiles(dd_plan_t plan, dd_dtype dtype, const dd_tiles *tiles);

@@ -33,7 +33,7 @@ EXPORTS = [
     "dd_selftest_wait_timeout", "dd_server_set_batch_window", "dd_unpack", "dd_detect",
     "dd_frontend", "dd_frontend_work_bytes", "dd_channelise", "dd_channelise_nspec",
     "dd_pfb_prototype", "dd_sync_noalloc", "dd_selftest_noalloc_timeout", "dd_add_peak",
-    "dd_execute_detect",
+    "dd_execute_detect", "dd_plan_groups",
 ]
 
 
@@ -88,6 +88,7 @@ def _load() -> ctypes.CDLL:
         "dd_plan_dmshift": (i32, [p, p]),
         "dd_plan_get_tiles": (i32, [p, i32, ctypes.POINTER(Tiles)]),
         "dd_plan_set_tiles": (i32, [p, i32, ctypes.POINTER(Tiles)]),
+        "dd_plan_groups": (i32, [p, i64]),
         "dd_execute": (i32, [p, p, i32, i64, i64, p, i64, i64, p]),
         "dd_execute_host": (i32, [p, p, i32, i64, i64, p, i64, i64]),
         "dd_execute_noalloc": (i32, [p, p, i32, i64, i64, p, i64, i64, p]),
@@ -376,6 +377,11 @@ class Plan:
                   words_per_thread=8):
         t = Tiles(dm_per_thread, dm_warps, time_warps, chan_per_stage, words_per_thread)
         check(lib.dd_plan_set_tiles(self.handle, dtype_code(dtype), ctypes.byref(t)))
+
+    def groups(self, nsamp_out: int) -> int:
+        """Channels per group of the kernel that execute would now run nsamp_out uint8 samples
+        in (0: the direct kernel, as while the plan's group table is not complete)."""
+        return lib.dd_plan_groups(self.handle, nsamp_out)
 
     # -- execution --------------------------------------------------------
     def execute_ptr(self, in_ptr: int, dtype: int, in_pitch: int, nsamp_in: int,

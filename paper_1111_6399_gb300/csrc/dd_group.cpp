@@ -264,6 +264,16 @@ void group_later(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &d
         group_start(p, dev, dt);
 }
 
+bool group_taken(dd_plan_s *p, dd_dtype t, const Geometry &g, int64_t nsamp_out,
+                 GroupShape *out) {
+    int dev = 0;
+    double gain = 0;
+    bool ready = false;
+    return may_group(t, g) && cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 &&
+           gains(p, dev, g, nsamp_out, &gain, &ready) && ready &&
+           group_ready(p, dev, DevTables(), false, out);
+}
+
 void group_free(dd_plan_s *p) {
     for (auto &kv : p->group) {
         cudaSetDevice(kv.first);
@@ -295,3 +305,14 @@ GroupBeam group_beam(const GroupShape &g, const DevTables &dt, const void *in, i
 }
 
 }  // namespace dd
+
+extern "C" int dd_plan_groups(dd_plan_t p, int64_t nsamp_out) {
+    int dev = 0;
+    dd::Geometry g;
+    dd::GroupShape gs;
+    if (!p || nsamp_out < 1 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 ||
+        !dd::group_sampled(p, dev) ||
+        dd::execution_geometry(p, DD_U8, nsamp_out, &g) != DD_OK)
+        return 0;
+    return dd::group_taken(p, DD_U8, g, nsamp_out, &gs) ? gs.G : 0;
+}

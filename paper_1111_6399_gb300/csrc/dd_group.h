@@ -196,6 +196,9 @@ constexpr double kGroupTableUs = 200.0;
 enum class GroupRoute { kDirect, kLater, kGrouped };
 GroupRoute group_route(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &dt,
                        int64_t nsamp_out, bool now, GroupShape *out);
+// Whether an execution would take the grouped kernel as things stand (*out).
+bool group_taken(dd_plan_s *p, dd_dtype t, const Geometry &g, int64_t nsamp_out,
+                 GroupShape *out);
 // After a kLater launch: start the table if the plan's next execution of this
 // length would take it.
 void group_later(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &dt,
