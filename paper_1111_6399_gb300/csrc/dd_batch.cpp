@@ -152,7 +152,8 @@ std::vector<int> grouped_beams(dd_batch_s *b, bool all, double *gain_us) {
 
 // Geometry, descriptors and launch shape for the current tiles.  Tables that
 // some beams would need and do not have are built first if `now` or if this
-// execution gains more than they cost; else all beams run directly and
+// execution gains more than they cost (started together, 80 us more for each
+// after the first); else all beams run directly and
 // b->tables names the beams whose tables are to be started behind the launch.
 dd_status prepare(dd_batch_s *b, bool now) {
     if (b->prepared)
@@ -202,12 +203,12 @@ dd_status prepare(dd_batch_s *b, bool now) {
     const int nsm = dd::sm_count(dev);
     double gain = 0;
     std::vector<int> grouped = grouped_beams(b, now, &gain), missing;
-    std::vector<dd::GroupShape> shapes(b->beams.size());
+    std::vector<dd::GroupTable> shapes(b->beams.size());
     for (int i : grouped)
         if (!dd::group_ready(b->beams[i].plan, dev, *tables[i], false, &shapes[i]))
             missing.push_back(i);
     b->tables.clear();
-    if (!missing.empty() && !now && gain <= dd::kGroupTableUs * (double)missing.size()) {
+    if (!missing.empty() && !now && gain <= dd::kGroupTableUs + 80.0 * (double)(missing.size() - 1)) {
         grouped.clear();
         b->tables = missing;
     } else {
@@ -225,7 +226,7 @@ dd_status prepare(dd_batch_s *b, bool now) {
             gdesc.push_back(dd::group_beam(shapes[i], *dt, bb.in, bb.in_pitch, bb.nsamp_in,
                                            bb.out, bb.out_pitch, bb.nsamp_out));
             gdesc.back().tile_begin = gtile0;
-            gtile0 += dd::group_tiles(shapes[i], bb.nsamp_out);
+            gtile0 += dd::group_tiles(shapes[i].ntile_d, bb.nsamp_out);
             continue;
         }
         desc.emplace_back();

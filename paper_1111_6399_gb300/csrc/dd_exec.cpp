@@ -244,9 +244,9 @@ extern "C" dd_status dd_execute_host(dd_plan_t p, const void *in_host, dd_dtype 
             return fail(DD_ERR_CUDA, std::string("input copy: ") + cudaGetErrorString(e));
         // A table for the blocks to come, while the first one's input is copied, if
         // all of them together gain more by it than it costs.
-        dd::GroupShape gs;
+        dd::GroupTable gs;
         if (k == 0)
-            dd::group_route(p, dtype, whole, *dt, nsamp_out, false, &gs);
+            dd::group_route(p, dtype, whole, *dt, nsamp_out, false, s, &gs);
         dd::Geometry g;
         if ((st = dd::execution_geometry(p, dtype, nb, &g)) != DD_OK)
             return st;

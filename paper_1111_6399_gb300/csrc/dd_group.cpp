@@ -128,7 +128,7 @@ GroupShape &shape_of(dd_plan_s *p, int dev) {
 }
 
 void start(dd_plan_s *p, int dev, const DevTables &dt, GroupShape &r) {
-    while (!r.entries && !r.build.entries && !r.sizes.empty()) {
+    while (!r.table.entries && !r.build.entries && !r.sizes.empty()) {
         GroupPrep a{};
         a.dmshift = dt.dmshift;
         a.dm_sorted = dt.dm_sorted;
@@ -159,9 +159,8 @@ void poll(dd_plan_s *p, int dev, GroupShape &r, bool wait) {
     if (st == TableState::kUnusable) {  // the sampled groups fitted, others do not
         r.sizes.erase(r.sizes.begin());
     } else if (st == TableState::kComplete) {
-        r.G = r.sizes[0].G;
-        r.npairs = ((p->nchan + r.G - 1) / r.G + 1) / 2;
-        r.entries = entries;
+        const int G = r.sizes[0].G;
+        r.table = {G, ((p->nchan + G - 1) / G + 1) / 2, r.ntile_d, r.rowcap, entries};
         r.sizes.resize(1);
     }
 }
@@ -177,19 +176,15 @@ bool may_group(dd_dtype t, const Geometry &g) {
     return t == DD_U8 && (g.chosen || std::memcmp(&pref, &g.tiles, sizeof(pref)) == 0);
 }
 
-// Times of an execution alone on the device, in rounds of tiles over the SMs.
-// False: the grouped form does not gain enough.
-bool gains(dd_plan_s *p, int dev, const Geometry &g, int64_t nsamp_out, double *gain_us,
-           bool *ready) {
+// Whether an execution alone on the device, of `direct` us by the direct kernel,
+// gains enough by groups: *grouped us, in rounds of tiles over the SMs.
+bool gains(dd_plan_s *p, int dev, double direct, int64_t nsamp_out, GroupEstimate *e,
+           double *grouped) {
     const int sms = sm_count(dev);
-    const double direct = sms > 0 ? direct_time_us(p, DD_U8, g.tiles, nsamp_out, sms) : -1.0;
-    GroupEstimate e;
-    if (direct < kLeastUs || !group_estimate(p, dev, nsamp_out, &e))
+    if (!group_estimate(p, dev, nsamp_out, e))
         return false;
-    const double grouped = (double)((e.tiles + sms - 1) / sms) * e.tile_us;
-    *gain_us = direct - grouped;
-    *ready = e.ready;
-    return grouped <= kGroupGain * direct;
+    *grouped = (double)((e->tiles + sms - 1) / sms) * e->tile_us;
+    return *grouped <= kGroupGain * direct;
 }
 
 }  // namespace
@@ -206,8 +201,8 @@ bool group_estimate(dd_plan_s *p, int dev, int64_t nsamp_out, GroupEstimate *e) 
     if (r.sizes.empty())
         return false;
     e->tile_us = tile_us(p, r);
-    e->tiles = group_tiles(r, nsamp_out);
-    e->ready = r.entries != nullptr;
+    e->tiles = group_tiles(r.ntile_d, nsamp_out);
+    e->ready = r.table.entries != nullptr;
     return true;
 }
 
@@ -216,37 +211,41 @@ void group_start(dd_plan_s *p, int dev, const DevTables &dt) {
     start(p, dev, dt, shape_of(p, dev));
 }
 
-bool group_ready(dd_plan_s *p, int dev, const DevTables &dt, bool now, GroupShape *out) {
+bool group_ready(dd_plan_s *p, int dev, const DevTables &dt, bool now, GroupTable *out) {
     std::lock_guard<std::mutex> lk(p->mu);
     GroupShape &r = shape_of(p, dev);
     poll(p, dev, r, now);
-    while (now && !r.entries && !r.sizes.empty()) {
+    while (now && !r.table.entries && !r.sizes.empty()) {
         start(p, dev, dt, r);
         poll(p, dev, r, true);
     }
-    if (!r.entries)
-        return false;
-    *out = r;
-    return true;
+    *out = r.table;
+    return out->entries != nullptr;
 }
 
 GroupRoute group_route(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &dt,
-                       int64_t nsamp_out, bool now, GroupShape *out) {
+                       int64_t nsamp_out, bool now, cudaStream_t stream, GroupTable *out) {
     int dev = 0;
     if (!may_group(t, g) || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
         return GroupRoute::kDirect;
-    if (!now && !group_sampled(p, dev)) {
-        const int sms = sm_count(dev);
-        const double direct = sms > 0 ? direct_time_us(p, t, g.tiles, nsamp_out, sms) : -1.0;
-        if (direct < kSampleUs)
-            return direct < kLeastUs ? GroupRoute::kDirect : GroupRoute::kLater;
-    }
-    double gain = 0;
-    bool ready = false;
+    const int sms = sm_count(dev);
+    const double direct = sms > 0 ? direct_time_us(p, t, g.tiles, nsamp_out, sms) : -1.0;
+    if (direct < kLeastUs)
+        return GroupRoute::kDirect;
+    auto captured = [&]() {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess)
+            cudaGetLastError();
+        return cap != cudaStreamCaptureStatusNone;
+    };
+    if (!now && direct < kSampleUs && !group_sampled(p, dev) && !(now = captured()))
+        return GroupRoute::kLater;
     // (Again if a table turns out unusable: another group size may serve.)
-    while (gains(p, dev, g, nsamp_out, &gain, &ready)) {
-        const bool wait = now || gain > kGroupTableUs;
-        if (!ready && !wait)
+    GroupEstimate e;
+    double grouped = 0;
+    while (gains(p, dev, direct, nsamp_out, &e, &grouped)) {
+        const bool wait = !e.ready && (now || direct - grouped > kGroupTableUs || captured());
+        if (!e.ready && !wait)
             return GroupRoute::kLater;
         if (group_ready(p, dev, dt, wait, out))
             return GroupRoute::kGrouped;
@@ -254,23 +253,30 @@ GroupRoute group_route(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTab
     return GroupRoute::kDirect;
 }
 
+// Whether it would be grouped if its table were there.
+static bool would_group(dd_plan_s *p, dd_dtype t, const Geometry &g, int64_t nsamp_out, int *dev,
+                        GroupEstimate *e) {
+    if (!may_group(t, g) || cudaGetDevice(dev) != cudaSuccess || *dev < 0 || *dev >= 64)
+        return false;
+    const int sms = sm_count(*dev);
+    const double direct = sms > 0 ? direct_time_us(p, t, g.tiles, nsamp_out, sms) : -1.0;
+    double grouped = 0;
+    return direct >= kLeastUs && gains(p, *dev, direct, nsamp_out, e, &grouped);
+}
+
 void group_later(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &dt,
                  int64_t nsamp_out) {
     int dev = 0;
-    double gain = 0;
-    bool ready = false;
-    if (may_group(t, g) && cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 &&
-        gains(p, dev, g, nsamp_out, &gain, &ready) && !ready)
+    GroupEstimate e;
+    if (would_group(p, t, g, nsamp_out, &dev, &e) && !e.ready)
         group_start(p, dev, dt);
 }
 
 bool group_taken(dd_plan_s *p, dd_dtype t, const Geometry &g, int64_t nsamp_out,
-                 GroupShape *out) {
+                 GroupTable *out) {
     int dev = 0;
-    double gain = 0;
-    bool ready = false;
-    return may_group(t, g) && cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 &&
-           gains(p, dev, g, nsamp_out, &gain, &ready) && ready &&
+    GroupEstimate e;
+    return would_group(p, t, g, nsamp_out, &dev, &e) && e.ready &&
            group_ready(p, dev, DevTables(), false, out);
 }
 
@@ -281,12 +287,12 @@ void group_free(dd_plan_s *p) {
         if (building &&
             finish_group_table(&kv.second->build, kv.first, true) == TableState::kComplete)
             cudaFree(building);
-        cudaFree(kv.second->entries);
+        cudaFree(kv.second->table.entries);
     }
     p->group.clear();
 }
 
-GroupBeam group_beam(const GroupShape &g, const DevTables &dt, const void *in, int64_t in_pitch,
+GroupBeam group_beam(const GroupTable &g, const DevTables &dt, const void *in, int64_t in_pitch,
                      int64_t nsamp_in, float *out, int64_t out_pitch, int64_t nsamp_out) {
     GroupBeam b{};
     b.in = static_cast<const uint8_t *>(in);
@@ -309,7 +315,7 @@ GroupBeam group_beam(const GroupShape &g, const DevTables &dt, const void *in, i
 extern "C" int dd_plan_groups(dd_plan_t p, int64_t nsamp_out) {
     int dev = 0;
     dd::Geometry g;
-    dd::GroupShape gs;
+    dd::GroupTable gs;
     if (!p || nsamp_out < 1 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 ||
         !dd::group_sampled(p, dev) ||
         dd::execution_geometry(p, DD_U8, nsamp_out, &g) != DD_OK)

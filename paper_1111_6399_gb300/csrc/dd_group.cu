@@ -21,16 +21,19 @@
 // A pair is built while the one before is used, in the other end of the array
 // space; mbarriers hand the arrays over, waits are bounded.
 //
-// Measured on the 4096-channel beam (2000 DMs x 262144 samples): 63.7 ms
+// Measured on the 4096-channel beam (2000 DMs x 262144 samples): 63.8 ms
 // against the direct kernel's 81.4; beams whose DM tiles span fewer samples
-// gain more (1024 channels over 64 MHz, 1024 DMs x 65536: 1.85 against 2.77).
-// The builders bound it: they are busy 80 % of the time, at 3 warps a
-// scheduler behind the users' shared-memory reads, and the users wait for
-// them 30 % of theirs.  Measured slower, on the same beam: 4 builder warps at
-// 128 registers (217 ms); 16 warps that build and use in turn, handing over by
-// mbarriers or a block barrier (68 - 72); 8 builder warps that also fetch
-// (68); 15 builders with 768-sample tiles (66.6).  FP16/FP32 forms of it (one
-// FP32 sum per group) did not beat the direct kernel's tuned tiles.
+// gain more (1024 channels over 64 MHz, 1024 DMs x 65536: 1.82 against 2.77).
+// No unit is full: on 16384 samples of that beam, issue slots 62 %, the
+// shared-memory pipe 73 %, ALU 53 % while CTAs are resident; a warp waits for
+// loads from shared memory (short scoreboard and MIO queue, 1.8 of 8.0 cycles an
+// instruction), for the fixed latency of its last instruction (1.6) or at a
+// hand-over (1.7, counted as long scoreboard).  Measured slower, on the same
+// beam: 4 builder warps at 128 registers (217 ms); 16 warps that build and use in
+// turn, handing over by mbarriers or a block barrier (68 - 72); 8 builder warps
+// that also fetch (68); 15 builders with 768-sample tiles (66.6).  Forms of it
+// for FP16/FP32 (one FP32 sum per group) were not kept: 40 - 60 ms against 37 on
+// that beam as FP16, 7.6 against 8.05 on the FP32 L-band beam.
 #include <cuda_runtime.h>
 
 #include <cstdint>

@@ -14,8 +14,8 @@
 //
 // This header: the tables that describe the patterns of every (DM tile,
 // group), built on the device once per plan (they do not depend on time,
-// because every tile starts at a multiple of 16 samples), and the arguments of
-// the kernel that uses them (dd_group.cu).
+// because every tile starts at a multiple of 16 samples; 2 KB per tile and pair of
+// groups), and the arguments of the kernel that uses them (dd_group.cu).
 #pragma once
 
 #include <cuda_runtime_api.h>
@@ -122,6 +122,12 @@ struct GroupBuild {
     cudaEvent_t done = nullptr;
 };
 
+// A complete table, as an execution uses it.
+struct GroupTable {
+    int G = 0, npairs = 0, ntile_d = 0, rowcap = 0;
+    GroupEntry *entries = nullptr;
+};
+
 // Grouped execution of a plan on one device.
 struct GroupShape {
     int ntile_d = 0, rowcap = 0;
@@ -133,8 +139,7 @@ struct GroupShape {
     };
     std::vector<Size> sizes;
     GroupBuild build;               // of sizes[0], under way if build.entries
-    int G = 0, npairs = 0;          // of the table
-    GroupEntry *entries = nullptr;  // device table, complete
+    GroupTable table;               // complete if table.entries
 };
 
 // Shared memory of a grouped CTA: kGroupRaw raw slots, then the array space.
@@ -179,7 +184,7 @@ bool group_estimate(dd_plan_s *p, int dev, int64_t nsamp_out, GroupEstimate *e);
 void group_start(dd_plan_s *p, int dev, const DevTables &dt);
 // The plan's grouped form, once its table is there: waited for, or started and
 // waited for (now), or left if not.
-bool group_ready(dd_plan_s *p, int dev, const DevTables &dt, bool now, GroupShape *out);
+bool group_ready(dd_plan_s *p, int dev, const DevTables &dt, bool now, GroupTable *out);
 
 // Grouped execution is taken when it is expected to gain this much: the model
 // is good to about 5 %.
@@ -191,24 +196,24 @@ constexpr double kGroupTableUs = 200.0;
 // How one execution by dd_execute runs: by the direct kernel, by the direct
 // kernel with the table to be started behind it (kGroupLater: the execution
 // would gain less than the table costs it), or by the grouped kernel (*out).
-// With `now` it waits for a table in any case (graph capture: the graph keeps
-// what it captures; the autotuner).
+// It waits for a table in any case with `now` (the autotuner) or while `stream`
+// is being captured (the graph keeps what it captures).
 enum class GroupRoute { kDirect, kLater, kGrouped };
 GroupRoute group_route(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &dt,
-                       int64_t nsamp_out, bool now, GroupShape *out);
+                       int64_t nsamp_out, bool now, cudaStream_t stream, GroupTable *out);
 // Whether an execution would take the grouped kernel as things stand (*out).
 bool group_taken(dd_plan_s *p, dd_dtype t, const Geometry &g, int64_t nsamp_out,
-                 GroupShape *out);
+                 GroupTable *out);
 // After a kLater launch: start the table if the plan's next execution of this
 // length would take it.
 void group_later(dd_plan_s *p, dd_dtype t, const Geometry &g, const DevTables &dt,
                  int64_t nsamp_out);
 void group_free(dd_plan_s *p);
 
-GroupBeam group_beam(const GroupShape &g, const DevTables &dt, const void *in, int64_t in_pitch,
+GroupBeam group_beam(const GroupTable &g, const DevTables &dt, const void *in, int64_t in_pitch,
                      int64_t nsamp_in, float *out, int64_t out_pitch, int64_t nsamp_out);
-inline int64_t group_tiles(const GroupShape &g, int64_t nsamp_out) {
-    return (nsamp_out + kGroupTCta - 1) / kGroupTCta * g.ntile_d;
+inline int64_t group_tiles(int ntile_d, int64_t nsamp_out) {
+    return (nsamp_out + kGroupTCta - 1) / kGroupTCta * ntile_d;
 }
 cudaError_t launch_group(const GroupArgs &a, unsigned grid, cudaStream_t s);
 

@@ -125,6 +125,14 @@ struct ShapeFit {
     int resident = 1;  // CTAs on an SM
 };
 
+struct ShapeChoice {
+    int64_t nsamp_out = -1;
+    int sms = 0;
+    uint32_t unfit = 0;
+    int place = -1;   // in the list of shapes
+    double us = 0;
+};
+
 }  // namespace dd
 
 struct dd_plan_s {
@@ -142,6 +150,7 @@ struct dd_plan_s {
     bool tiles_open[3] = {true, true, true};  // executions may choose, until set
     std::map<uint64_t, dd::Geometry> geo;  // per (dtype, tiles) key
     std::vector<dd::ShapeFit> shape_fit[3];  // of the listed shapes (dd_shape.cpp), on first use
+    dd::ShapeChoice shape_choice[3];         // for the last length asked for
     float most_delay = -1.0f;                // of dmshift, with the first of those
     uint32_t shape_unfit[3] = {0, 0, 0};     // shapes found not to fit, a bit each
     // Remainder-DM launch per (dtype, tiles) key: (found, geometry).

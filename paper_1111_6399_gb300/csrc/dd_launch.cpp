@@ -165,18 +165,14 @@ dd_status launch_dedisperse(dd_plan_s *p, const Geometry &g, const DevTables &dt
                             bool split_tail, Grouped grouped) {
     if (nsamp_out == 0)
         return DD_OK;
-    GroupShape gs;
+    GroupTable gs;
     GroupRoute route = GroupRoute::kDirect;
-    if (grouped != Grouped::kNever && dtype == DD_U8) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) != cudaSuccess)
-            cudaGetLastError();
-        route = group_route(p, dtype, g, dt, nsamp_out,
-                            grouped == Grouped::kNow || cap != cudaStreamCaptureStatusNone, &gs);
-    }
+    if (grouped != Grouped::kNever)
+        route = group_route(p, dtype, g, dt, nsamp_out, grouped == Grouped::kNow,
+                            static_cast<cudaStream_t>(stream), &gs);
     if (route == GroupRoute::kGrouped) {
         cudaStream_t s = static_cast<cudaStream_t>(stream);
-        const int64_t tiles = group_tiles(gs, nsamp_out);
+        const int64_t tiles = group_tiles(gs.ntile_d, nsamp_out);
         if (tiles > 0x7fffffffLL)
             return fail(DD_ERR_INVALID, "too many tiles for one launch");
         GroupArgs a{};

@@ -175,6 +175,11 @@ int place_of(dd_dtype t, const dd_tiles &tl) {
 // The listed shape expected to finish first (-1: none fits), and its time.
 // Caller holds p->mu.
 int fastest_shape(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, int sms, double *us) {
+    ShapeChoice &last = p->shape_choice[t];
+    if (last.nsamp_out == nsamp_out && last.sms == sms && last.unfit == p->shape_unfit[t]) {
+        *us = last.us;
+        return last.place;
+    }
     const std::vector<ShapeCost> &shapes = shape_costs(t);
     const bool narrow = shape_fit(p, t, 0).stages >= 3;
     int best = -1;
@@ -191,6 +196,7 @@ int fastest_shape(dd_plan_s *p, dd_dtype t, int64_t nsamp_out, int sms, double *
             *us = u;
         }
     }
+    last = {nsamp_out, sms, p->shape_unfit[t], best, *us};
     return best;
 }
 
