@@ -51,50 +51,59 @@ TUNE_NSAMP = 65536
 
 # DRAM traffic of one de-dispersion step from an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum of its launches), valid only
-# for the kernel and launch code it was taken on (sha256 of csrc/dd_kernel.cuh
-# and csrc/dd_launch.cpp) and the same workload, dtype and tile shape; any
-# other run reports traffic null.
+# for the kernel and launch code it was taken on (sha256 of the sources named
+# below and the headers that they include) and the same workload, dtype and tile
+# shape, or for steps in the channel-group kernel the same channels per group;
+# any other run reports traffic null.
 TRAFFIC_SOURCE = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum "
                   "--clock-control none, one step's de-dispersion launches")
 PROFILED_TRAFFIC: list[dict] = [
-    # one step, 4096-channel beam, tiles (4,12,1,8,8): a single launch of 42 x 256 tiles
-    {"workload": "lowfreq-4096ch-2000dm-262144", "dtype": "u8", "tiles": [4, 12, 1, 8, 8],
-     "code_sha256": "81b799d99197287efbc40fdfa738662c596bf5a398684d03d44737ff4d1d8816",
-     "bytes": 4790403072 + 2875413504, "compulsory": 1203281920 + 2097152000},
-    # one step, the same beam stored as FP16, tiles (4,12,1,12,8): a single launch
-    {"workload": "lowfreq-4096ch-2000dm-262144", "dtype": "f16", "tiles": [4, 12, 1, 12, 8],
-     "code_sha256": "81b799d99197287efbc40fdfa738662c596bf5a398684d03d44737ff4d1d8816",
-     "bytes": 20705216768 + 2230952960, "compulsory": 2406563840 + 2097152000},
-    # one step, the same beam stored as FP32, tiles (4,6,2,24,8): main launch (1992 DMs) +
-    # remainder (8 DMs)
-    {"workload": "lowfreq-4096ch-2000dm-262144", "dtype": "f32", "tiles": [4, 6, 2, 24, 8],
-     "code_sha256": "81b799d99197287efbc40fdfa738662c596bf5a398684d03d44737ff4d1d8816",
-     "bytes": (86389575424 + 2099985408) + (4307168768 + 7886080),
-     "compulsory": 4813127680 + 2097152000},
-    # one step, L-band beam, tiles (4,12,1,8,8): main launch (1008 DMs) + remainder (16 DMs)
-    {"workload": "lband-1024ch-1024dm-131072", "dtype": "u8", "tiles": [4, 12, 1, 8, 8],
-     "code_sha256": "81b799d99197287efbc40fdfa738662c596bf5a398684d03d44737ff4d1d8816",
-     "bytes": (153392640 + 506828544) + (135646464 + 358912),
-     "compulsory": 151171072 + 536870912},
 ]
+PROFILED_GROUP_TRAFFIC: list[dict] = [
+]
+GROUP_SOURCES = ("dd_group.cu", "dd_group.cpp")
 
 
 def _sha256(*parts) -> str:
+    """Of sources under csrc/ and the headers there that they include."""
     import hashlib
+    import re
     h = hashlib.sha256()
-    for rel in parts:
-        with open(os.path.join(ROOT, "paper_1111_6399_gb300", "csrc", rel), "rb") as f:
-            h.update(hashlib.sha256(f.read()).digest())
+    todo, seen = list(parts), set()
+    while todo:
+        rel = todo.pop(0)
+        if rel in seen:
+            continue
+        seen.add(rel)
+        path = os.path.join(ROOT, "paper_1111_6399_gb300", "csrc", rel)
+        if not os.path.exists(path):  # the public header, beside csrc/
+            continue
+        with open(path, "rb") as f:
+            data = f.read()
+        h.update(hashlib.sha256(data).digest())
+        todo += re.findall(r'#include "([^"]+)"', data.decode())
     return h.hexdigest()
 
 
-def profiled_traffic(workload: str, dtype: str, tiles) -> dict | None:
+def profiled_traffic(workload: str, dtype: str, tiles, groups: int = 0) -> dict | None:
+    if groups:
+        digest = _sha256(*GROUP_SOURCES)
+        for rec in PROFILED_GROUP_TRAFFIC:
+            if (rec["code_sha256"] == digest and rec["workload"] == workload
+                    and rec["groups"] == groups):
+                return rec
+        return None
     digest = _sha256("dd_kernel.cuh", "dd_launch.cpp")
     for rec in PROFILED_TRAFFIC:
         if (rec["code_sha256"] == digest and rec["workload"] == workload
                 and rec["dtype"] == dtype and list(rec["tiles"]) == list(tiles)):
             return rec
     return None
+
+
+def step_groups(plan, dtype: str, nsamp_out: int) -> int:
+    """Channels per group if the plan's steps run in the channel-group kernel, else 0."""
+    return plan.groups(nsamp_out) if dtype == "u8" else 0
 
 
 def peaks():
@@ -770,9 +779,9 @@ def e2e_rate(plan, host, nin: int, w: fb.Workload, torch, reps: int, barrier) ->
 
 
 def roofline_of(adds: float, kernel_ms: float, peak: dict, nominal: float, w: fb.Workload,
-                dtype: str, tiles, traffic_ok: bool = True) -> dict:
+                dtype: str, tiles, traffic_ok: bool = True, groups: int = 0) -> dict:
     achieved = adds / (kernel_ms / 1e3)
-    prof = profiled_traffic(w.name, dtype, tiles) if traffic_ok else None
+    prof = profiled_traffic(w.name, dtype, tiles, groups) if traffic_ok else None
     return {"bound": "alu", "achieved": achieved / 1e12, "peak": peak["adds_per_s"] / 1e12,
             "traffic_over_compulsory": prof["bytes"] / prof["compulsory"] if prof else None,
             "unit": "Tadd/s", "frac": achieved / peak["adds_per_s"],
@@ -782,8 +791,12 @@ def roofline_of(adds: float, kernel_ms: float, peak: dict, nominal: float, w: fb
             "traffic": prof["bytes"] if prof else None,
             "traffic_unit": "bytes per step (ncu dram read + write of its launches)",
             "traffic_source": TRAFFIC_SOURCE if prof else None,
-            "kernel": "dedisperse_kernel<%d,%d,%d>" % ({"u8": 1, "f16": 2, "f32": 4}[dtype],
-                                                       tiles[0], tiles[4]),
+            "adds": ("the definition's; the channel-group kernel sums %d channels once per "
+                     "shift pattern and performs fewer" % groups) if groups
+            else "the definition's, all performed",
+            "kernel": "group_kernel (%d channels a group)" % groups if groups
+            else "dedisperse_kernel<%d,%d,%d>" % ({"u8": 1, "f16": 2, "f32": 4}[dtype],
+                                                  tiles[0], tiles[4]),
             "kernel_ms": kernel_ms}
 
 
@@ -806,7 +819,8 @@ def beam_section(dd, torch, dev, w: fb.Workload, dtype: str, steps: int, warmup:
                                                   warmup, barrier)
     step_ms = sum(per_step) / len(per_step)
     tiles = plan.get_tiles(dtype)
-    rl = roofline_of(w.adds(), kernel_ms, peak, nominal, w, dtype, tiles)
+    rl = roofline_of(w.adds(), kernel_ms, peak, nominal, w, dtype, tiles,
+                     groups=step_groups(plan, dtype, w.nsamp_out))
     rl["compulsory_bytes"] = int(w.nchan * nin * host.itemsize + w.ndm * w.nsamp_out * 4)
     del x, out
     torch.cuda.empty_cache()
@@ -874,7 +888,8 @@ def run_ours(args, w):
         dist.destroy_process_group()
         return
     clocks = clk.summary()
-    rl = roofline_of(adds, kernel_ms, peak, nominal, w, dt, tiles)
+    rl = roofline_of(adds, kernel_ms, peak, nominal, w, dt, tiles,
+                     groups=step_groups(plan, dt, w.nsamp_out))
     rl["compulsory_bytes"] = int(w.nchan * nin * host.itemsize + w.ndm * w.nsamp_out * 4)
     rl["step_ms"] = step_ms
     line = {
@@ -978,7 +993,8 @@ def sweep(dd, torch, dev, compact: bool = False) -> dict:
         adds = nchan * ndm * nsamp_out
         return {"nchan": nchan, "ndm": ndm, "max_dm": maxdm, "maxshift": plan.maxshift,
                 "ms": ms, "pct_real_time": 100.0 * ms / 1e3 / duration,
-                "adds_per_s": adds / ms * 1e3, "tiles": plan.get_tiles("u8")}
+                "adds_per_s": adds / ms * 1e3, "tiles": plan.get_tiles("u8"),
+                "groups": plan.groups(nsamp_out)}
 
     nchans = (512, 2048, 4096) if compact else (128, 256, 512, 1024, 2048, 4096)
     maxdms = (100.0, 400.0, 1600.0) if compact else (50.0, 100.0, 200.0, 400.0, 800.0, 1600.0)

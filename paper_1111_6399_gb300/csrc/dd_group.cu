@@ -24,11 +24,11 @@
 // Measured on the 4096-channel beam (2000 DMs x 262144 samples): 63.8 ms
 // against the direct kernel's 81.4; beams whose DM tiles span fewer samples
 // gain more (1024 channels over 64 MHz, 1024 DMs x 65536: 1.82 against 2.77).
-// No unit is full: on 16384 samples of that beam, issue slots 62 %, the
-// shared-memory pipe 73 %, ALU 53 % while CTAs are resident; a warp waits for
-// loads from shared memory (short scoreboard and MIO queue, 1.8 of 8.0 cycles an
-// instruction), for the fixed latency of its last instruction (1.6) or at a
-// hand-over (1.7, counted as long scoreboard).  Measured slower, on the same
+// No unit is full: on 16384 samples of that beam, issue slots 62 %, L1 and shared
+// memory 73 %, ALU 53 % while CTAs are resident.  Of 8.0 cycles an instruction,
+// a warp waits 1.8 for shared-memory loads and their queue, 1.7 on a long
+// scoreboard (in the loops only the hand-overs and the fetch warp's records have
+// one), 1.6 for the latency of the instruction before.  Measured slower, on the same
 // beam: 4 builder warps at 128 registers (217 ms); 16 warps that build and use in
 // turn, handing over by mbarriers or a block barrier (68 - 72); 8 builder warps
 // that also fetch (68); 15 builders with 768-sample tiles (66.6).  Forms of it
