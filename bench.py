@@ -58,8 +58,27 @@ TUNE_NSAMP = 65536
 TRAFFIC_SOURCE = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum "
                   "--clock-control none, one step's de-dispersion launches")
 PROFILED_TRAFFIC: list[dict] = [
+    # one step, the 4096-channel beam stored as FP16, tiles (4,12,1,12,8): a single launch
+    {"workload": "lowfreq-4096ch-2000dm-262144", "dtype": "f16", "tiles": [4, 12, 1, 12, 8],
+     "code_sha256": "938ed6f837933cf8b21255ba85f3cf99b19435026f7a7fac7a47ff362ab8fafa",
+     "bytes": 24604479744 + 2231196928, "compulsory": 2406563840 + 2097152000},
+    # one step, the same beam stored as FP32, tiles (4,6,2,24,8): main launch (1992 DMs) +
+    # remainder (8 DMs)
+    {"workload": "lowfreq-4096ch-2000dm-262144", "dtype": "f32", "tiles": [4, 6, 2, 24, 8],
+     "code_sha256": "938ed6f837933cf8b21255ba85f3cf99b19435026f7a7fac7a47ff362ab8fafa",
+     "bytes": (103365352192 + 2099205888) + (4306778112 + 7870720),
+     "compulsory": 4813127680 + 2097152000},
+    # one step, L-band beam, tiles (4,12,1,8,8): main launch (1008 DMs) + remainder (16 DMs)
+    {"workload": "lband-1024ch-1024dm-131072", "dtype": "u8", "tiles": [4, 12, 1, 8, 8],
+     "code_sha256": "938ed6f837933cf8b21255ba85f3cf99b19435026f7a7fac7a47ff362ab8fafa",
+     "bytes": (153793024 + 507151104) + (135693824 + 142848),
+     "compulsory": 151171072 + 536870912},
 ]
 PROFILED_GROUP_TRAFFIC: list[dict] = [
+    # one step, 4096-channel beam: a single launch of 32 x 256 tiles
+    {"workload": "lowfreq-4096ch-2000dm-262144", "groups": 4,
+     "code_sha256": "23264bb0c89a0575959e6adae562acb798cf7226837f71cb5279ec9a1be69cb3",
+     "bytes": 17152169216 + 8343288320, "compulsory": 1203281920 + 2097152000},
 ]
 GROUP_SOURCES = ("dd_group.cu", "dd_group.cpp")
 
