@@ -164,3 +164,36 @@ def test_that_batch_takes_the_group_kernel():
         assert host.batch_execute(batch) == 0
     assert [r.beams for r in host.records(hostrt.GROUPED)] == [4, 4]
     assert host.records(hostrt.DIRECT)[-1].beams == 1
+
+
+@pytest.mark.gpu
+def test_threads_share_a_plan_whose_table_is_under_way(built_lib):
+    """Four threads, each with a stream and an output of its own, from the first
+    execution on: some take the direct kernel, later ones the group kernel."""
+    import threading
+
+    import torch
+    nchan, top, width, ndm, lo, step, ns, G = CASES[3]
+    plan = built_lib.Plan(nchan, top, width, TSAMP, _dms(ndm, lo, step))
+    nin = ns + plan.maxshift
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    x = torch.randint(0, 256, (nchan, (nin + 15) // 16 * 16), dtype=torch.uint8, device="cuda",
+                      generator=gen)
+    outs = [torch.zeros((8, ndm, (ns + 3) // 4 * 4), device="cuda") for _ in range(4)]
+    streams = [torch.cuda.Stream() for _ in outs]
+    torch.cuda.synchronize()
+
+    def work(out, stream):
+        for k in range(len(out)):
+            plan.execute(x, out[k], nsamp_in=nin, nsamp_out=ns, stream=stream)
+
+    threads = [threading.Thread(target=work, args=a) for a in zip(outs, streams)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    plan.sync(torch.cuda.current_stream())
+    assert plan.groups(ns) == G
+    for out in outs:
+        assert bool((out[:, :, :ns] == outs[0][0, :, :ns]).all())
