@@ -334,6 +334,11 @@ void look_after_tables(dd_batch_s *b) {
         drop_graph(b);
 }
 
+// De-dispersion kernels of one execution.
+int launches(const dd_batch_s *b) {
+    return (b->args.nbeams > 0 ? 1 : 0) + (b->gargs.nbeams > 0 ? 1 : 0);
+}
+
 // The tile counter reset and the persistent launch of the direct beams; the
 // grouped beams' launch beside it.
 dd_status enqueue(dd_batch_s *b, cudaStream_t s, bool count = true) {
@@ -369,7 +374,7 @@ dd_status enqueue(dd_batch_s *b, cudaStream_t s, bool count = true) {
     if (e != cudaSuccess)
         return fail(DD_ERR_CUDA, std::string("batch kernel launch: ") + cudaGetErrorString(e));
     if (count)
-        dd::count_launch((direct ? 1 : 0) + (grouped ? 1 : 0));
+        dd::count_launch(launches(b));
     return DD_OK;
 }
 
@@ -509,7 +514,7 @@ dd_status dd_batch_execute(dd_batch_t b, void *stream) {
     cudaError_t e = cudaGraphLaunch(b->exec, s);
     if (e != cudaSuccess)
         return fail(DD_ERR_CUDA, std::string("graph launch: ") + cudaGetErrorString(e));
-    dd::count_launch((int)(b->dtype == DD_F32 ? 1 : b->beams.size() + 1));
+    dd::count_launch(launches(b));
     return DD_OK;
 }
 

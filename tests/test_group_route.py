@@ -135,3 +135,17 @@ def test_batch_with_unusable_tables(host):
         assert host.batch_execute(batch) == 0
     launches = host.records(DIRECT, GROUPED)
     assert {r.kind for r in launches} == {DIRECT} and not any(r.null_pointers for r in launches)
+
+
+@pytest.mark.parametrize("kind", ["u8", "f16", "f32"])
+def test_a_replayed_batch_counts_the_kernels_that_its_graph_holds(host, kind):
+    """dd_launch_count: the same for the eager execution as for the graph's."""
+    plans = [_narrow(host, 1024, 1024), _lband(host, 64, 40), _lband(host, 64, 40)]
+    batch = host.batch(plans, kind, [65536, 8192, 8192])
+    host.lib.dd_launch_count.restype = hostrt.ctypes.c_int64
+    counts = []
+    for _ in range(3):
+        before = host.lib.dd_launch_count()
+        assert host.batch_execute(batch) == 0
+        counts.append(host.lib.dd_launch_count() - before)
+    assert counts == 3 * [2 if kind == "u8" else 1]
